@@ -209,10 +209,10 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
 int fdph_step(fdph_plan_t plan, const double* D_n, double* T_n);
 
 /* `steps` consecutive steps: D (device, steps * n doubles, step-major) -> T (device, same shape).
- * Equivalent to `steps` calls of fdph_step; from 8 steps on (and with profiling off) the call
- * replays a CUDA graph of one step, which removes the per-kernel launch cost; the graph is kept
- * with the plan (at most 8 per plan) and reused by later calls on the same D, T buffers.
- * Errors as fdph_step; FDPH_E_STATE if the plan would pass step M. */
+ * Equivalent to `steps` calls of fdph_step, bit for bit: the steps run in blocks of up to 16, each
+ * kernel one launch per block, so that the operator is read once per block; every output is summed
+ * in the order of the single step.  D == T is allowed (each block reads its rows before it writes
+ * them); rows that overlap in another way are taken one step at a time.  Errors as fdph_step; FDPH_E_STATE if the plan would pass step M. */
 int fdph_run(fdph_plan_t plan, int32_t steps, const double* D, double* T);
 
 /* Dynamic rupture (Sec. 6.2): the slip rate is not prescribed but follows from a friction law
@@ -242,9 +242,11 @@ int fdph_rupture_init(fdph_plan_t plan, const fdph_friction* friction);
  * tau0 + T_n (both device, n doubles, geometry order) and advances to n + 1. */
 int fdph_rupture_step(fdph_plan_t plan, double* D_n, double* T_n);
 
-/* `steps` rupture steps into D, T (device, steps * n doubles, step-major).  From 8 steps on
- * (profiling off) one rupture step is captured as a CUDA graph and replayed; the graph is kept
- * with the plan for later calls on the same D, T buffers. */
+/* `steps` rupture steps into D, T (device, steps * n doubles, step-major), bit for bit those of
+ * fdph_rupture_step: what the slip rates before a block of 16 steps (n rounded down to a multiple of
+ * 16) do to the block is computed at once, the block's own part step by step.  In calls of 8 steps and
+ * more (profiling off) a whole block is captured as a CUDA graph and replayed; the graph is kept with
+ * the plan for later calls on the same D, T buffers (at most 8 per plan). */
 int fdph_rupture_run(fdph_plan_t plan, int32_t steps, double* D, double* T);
 
 /* Copy the accumulated slip (device, n doubles, geometry order). */
@@ -266,24 +268,21 @@ int fdph_predict(fdph_plan_t plan, double* T_pred);
 int fdph_commit(fdph_plan_t plan, const double* D_n);
 
 /* Batches (no counterpart in the paper; the serving pattern of independent scenarios): plans
- * that share the device and the precision, stepped together.  Every kernel of a batch step is
- * ONE launch over the work of all plans: push, FIR and scatter (Eqs. 32, 42), transient and
- * Eq. 39 over the concatenated elements and warp tasks, and the persistent near-field kernel
- * (App. E) over the work items of all plans, dealt largest first over the SMs; the step is
- * captured once per (kind, buffers) as a CUDA graph and replayed.  Each plan keeps its own state
- * and step index, and its results are bit-identical to stepping it alone.
+ * that share the device and the precision, stepped together, each plan's blocks of steps on its own
+ * stream beside those of the others.  Each plan keeps its own state and step index, and its results
+ * are bit-identical to stepping it alone.
  *
  * fdph_batch_create: `plans` (count >= 1, distinct, host array, copied) must outlive the batch.
  *   Errors: FDPH_E_ARG (null, duplicate, mixed device or precision), FDPH_E_STATE (a predict
  *   pending), FDPH_E_CUDA.  fdph_autotune on a member plan invalidates the batch (later batch
  *   calls return FDPH_E_STATE; create it again).
  * fdph_batch_run: `steps` steps of every plan; D[p], T[p] (host arrays of device pointers):
- *   plan p's rows, steps * n_p doubles, step-major, as fdph_run.  Asynchronous; every plan's
- *   stream is ordered after the batch's work.  Errors as fdph_run for any plan.
+ *   plan p's rows, steps * n_p doubles, step-major, as fdph_run.  Asynchronous on the plans'
+ *   streams.  Errors as fdph_run for any plan.
  * fdph_batch_rupture_run: the same for rupture steps (fdph_rupture_init on every plan) with the
  *   outputs of fdph_rupture_run.
- * fdph_batch_synchronize: wait for the batch and its plans; reports a near-field wait that gave
- *   up (FDPH_E_TIMEOUT).  fdph_batch_destroy: release the batch (not its plans); NULL ignored. */
+ * fdph_batch_synchronize: wait for the batch's plans; reports a device error (as
+ *   fdph_synchronize).  fdph_batch_destroy: release the batch (not its plans); NULL ignored. */
 int fdph_batch_create(const fdph_plan_t* plans, int32_t count, fdph_batch_t* out);
 int fdph_batch_run(fdph_batch_t batch, int32_t steps, const double* const* D, double* const* T);
 int fdph_batch_rupture_run(fdph_batch_t batch, int32_t steps, double* const* D, double* const* T);
@@ -301,25 +300,22 @@ int fdph_step_host(fdph_plan_t plan, const double* D_n_host, double* T_n_host);
 
 /* `steps` consecutive steps with HOST buffers: D_host (steps * n doubles, step-major) ->
  * T_host (same shape).  Every step's D_n is copied to the device and its T_n back to the host
- * (page-locked buffers let the copies run asynchronously); the copies of later and earlier steps
- * overlap the step in progress through a ring of device staging slots, and the steps replay
- * one captured step graph.  Returns when T_host is complete.  Errors as fdph_run. */
+ * (page-locked buffers let the copies run asynchronously); the copies of later and earlier blocks
+ * overlap the block of steps in progress through a ring of device staging slots.  Returns when T_host is complete.  Errors as fdph_run. */
 int fdph_run_host(fdph_plan_t plan, int32_t steps, const double* D_host, double* T_host);
 
-/* Self-test of the device-side timeout path (no counterpart in the paper): every wait of the
- * library's pipelines polls an mbarrier a bounded number of times and, if it gives up, records
- * the fact and lets the kernel finish, after which the host call returns FDPH_E_TIMEOUT and the
- * CUDA context stays usable.  This call runs one such wait, with `polls` in [1, 2^24], on a
+/* Self-test of the device-side timeout path (no counterpart in the paper): a wait in a
+ * kernel polls an mbarrier a bounded number of times and, if it gives up, records the fact and lets
+ * the kernel finish, after which the host call returns FDPH_E_TIMEOUT and the CUDA context stays
+ * usable.  This call runs one such wait, with `polls` in [1, 2^24], on a
  * barrier that nothing completes, on `device`.  Returns FDPH_E_TIMEOUT when the path works,
  * FDPH_E_ARG for an out-of-range `polls`, FDPH_E_CUDA on a CUDA error. */
 int fdph_selftest_wait_timeout(int32_t device, int64_t polls);
 
-/* Autotuner of the near-field work items (no counterpart in the paper): times `steps` replayed
+/* Autotuner of the near-field work items (no counterpart in the paper): times `steps`
  * steps (1..1024; plan's M >= steps + 2) at a steady-state step index for work items of 64, 32
  * and 16 kernel steps (divided by nrhs unless the tensor cores take them), keeps the fastest and
- * writes it to *chunk (may be NULL); then times the other form of the Eq. 32 FIR (source-major,
- * the default where the F blocks hold each source ~100 times or more, or sub-block-major; both
- * give the same bits) and keeps the faster.  The plan's state and step index are saved and
+ * writes it to *chunk (may be NULL).  The plan's state and step index are saved and
  * restored, so results continue as before (summation order within the near field may change:
  * rounding-level differences).  Cached step graphs are dropped.
  * Errors: FDPH_E_ARG, FDPH_E_STATE (profiling on), FDPH_E_OOM, FDPH_E_CUDA. */
@@ -356,7 +352,7 @@ void fdph_destroy(fdph_plan_t plan);
 /* Per-kernel timing with CUDA events on the plan's stream (off by default).  Kernel ids:
  * 0 push, 1 fir (Eq. 32), 2 scatter (Eq. 42), 3 transient convolution (App. B.3),
  * 4 near field (App. E), 5 gather (Eq. 39).  fdph_kernel_times synchronises the stream and
- * returns, per id, the summed milliseconds and the launch count since profiling was enabled
+ * returns, per id, the summed milliseconds and the number of steps they cover since profiling was enabled
  * (arrays of length FDPH_NUM_KERNELS).  Enabling resets the counters. */
 #define FDPH_NUM_KERNELS 6
 int fdph_set_profiling(fdph_plan_t plan, int enable);

@@ -457,10 +457,10 @@ int build_host_far(const Elements& el, const PlanInputs& in, HostPlan& hp) {
             hp.ustate_len += (int64_t)sb.rank * (soe + sb.qn);
             if (kind == SB_TR) {
                 // + the input Y(t - taps) of the tail and of the last running sum
-                sb.L = sb.maxdelay + mindm + taps + (soe || sb.qn ? 1 : 0);
-                sb.LZ = maxdm - mindm + 1 + ex;
+                sb.L = sb.maxdelay + mindm + taps + (soe || sb.qn ? 1 : 0) + kRingRoom;
+                sb.LZ = maxdm - mindm + 1 + ex + kRingRoom;
             } else {
-                sb.L = sb.maxdelay + maxdm + 1 + ex;
+                sb.L = sb.maxdelay + maxdm + 1 + ex + kRingRoom;
                 sb.LZ = 0;
             }
             sb.ring = hp.ring_len;
@@ -557,8 +557,8 @@ int build_host_far(const Elements& el, const PlanInputs& in, HostPlan& hp) {
     return 0;
 }
 
-void finish_near_layout(HostPlan& hp, const std::vector<int32_t>& W, const std::vector<char>& has_tail, int chunk,
-                        int vec, int vec_aux, int aux_chunk) {
+void finish_near_layout(HostPlan& hp, const std::vector<int32_t>& W, const std::vector<int32_t>& kz,
+                        const std::vector<char>& has_tail, int chunk, int vec, int vec_aux, int aux_chunk) {
     const int nl = (int)hp.near_r0.size();
     hp.near.resize(nl);
     hp.items.clear();
@@ -575,6 +575,7 @@ void finish_near_layout(HostPlan& hp, const std::vector<int32_t>& W, const std::
         L.s0 = hp.near_s0[l];
         L.ns = hp.near_ns[l];
         L.W = W[l];
+        L.kz = kz[l];
         L.sl = (L.ns + vec - 1) / vec * vec * L.nr;
         L.sla = (L.ns + vec_aux - 1) / vec_aux * vec_aux * L.nr;
         L.tensor = hp.near_tensor_len;                     // stays a multiple of vec elements
@@ -603,7 +604,7 @@ void finish_near_layout(HostPlan& hp, const std::vector<int32_t>& W, const std::
             hp.items.push_back(it);
             for (int il = 0; il < L.nr; ++il) slots[L.r0 + il].push_back(id * 32 + il);
         };
-        for (int k0 = 0; k0 < L.W; k0 += chunk) add(0, k0, std::min(L.W, k0 + chunk));
+        for (int k0 = L.kz; k0 < L.W; k0 += chunk) add(0, k0, std::min(L.W, k0 + chunk));
         for (int k0 = 0; k0 < L.naux; k0 += aux_chunk) add(1, k0, std::min(L.naux, k0 + aux_chunk));
     }
     hp.np_ptr.assign(hp.n + 1, 0);

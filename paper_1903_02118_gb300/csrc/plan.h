@@ -8,14 +8,18 @@
 
 namespace fdph {
 
+// Ring slots beyond what one step needs, so that a block of up to kRingRoom + 1 steps can run at once
+static const int kRingRoom = 15;
+
 enum SubKind { SB_F = 0, SB_S = 1, SB_TR = 2 };
 
 // One low-rank operator: admissible leaf x domain (F / S / transient) x stress component.
 // Receivers [r0, r0 + nr), sources [s0, s0 + ns) in internal order.
 struct SubBlock {
     int32_t kind, rank, r0, nr, s0, ns;
-    int32_t L;         // ring length (F, S: representative-stress ring; TR: source-sum ring Y)
-    int32_t LZ;        // TR: length of the convolved ring Z
+    int32_t L;         // ring length (F, S: representative-stress ring; TR: source-sum ring Y), kRingRoom
+                       // slots of it beyond what one step needs
+    int32_t LZ;        // TR: length of the convolved ring Z (with the same room)
     int32_t taps;      // F: waveform taps (max Dm of the leaf); TR: Dm_tr
     int32_t maxdelay, mindelay, mindm, maxdm;
     int64_t f, g, h;   // offsets into the factor array (f: nr x rank, g: ns x rank, h: taps x ns or taps)
@@ -35,6 +39,7 @@ struct SubBlock {
 
 struct NearLeaf {
     int32_t r0, nr, s0, ns, W;   // W = window of exact kernel steps stored
+    int32_t kz;                  // leading steps of the window whose kernel vanishes (no work item covers them)
     // Slices are stored source-interleaved: element (j, i) of a slice at ((j / v) * nr + i) * v + j % v
     // with v = 16 bytes / element size, the sources padded with zeros to a multiple of v, so that a
     // receiver reads v sources with one 16-byte load.
@@ -108,8 +113,8 @@ int check_causality(const Elements& el, const PlanInputs& in, const Tree& tr);
 int build_host_far(const Elements& el, const PlanInputs& in, HostPlan& hp);
 // Second stage once the near-field windows W are known (fills offsets, items, CSR).
 // vec, vec_aux: sources per 16 bytes of the window and aux storage types (8 FP16, 4 FP32, 2 FP64);
-// chunk, aux_chunk: window and aux slices per work item at most.
-void finish_near_layout(HostPlan& hp, const std::vector<int32_t>& W, const std::vector<char>& has_tail, int chunk,
-                        int vec, int vec_aux, int aux_chunk);
+// chunk, aux_chunk: window and aux slices per work item at most; kz: leading window steps that vanish.
+void finish_near_layout(HostPlan& hp, const std::vector<int32_t>& W, const std::vector<int32_t>& kz,
+                        const std::vector<char>& has_tail, int chunk, int vec, int vec_aux, int aux_chunk);
 
 }  // namespace fdph
