@@ -9,6 +9,7 @@
 // that loads the library until the process exits.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -18,8 +19,9 @@
 namespace {
 
 const int kTile = 32;          // receivers per work item
-const int kSteps = 64;         // kernel steps per work item
-const int kThreads = 128;
+const int kSteps = 64;         // kernel steps per work item of the documented size limit
+const int kWarps = 8;
+const int kThreads = 32 * kWarps;
 
 // Shared by every call on a device; each call overwrites the slots it uses.
 static __device__ __align__(256) double g_noalloc_partials[FDPH_NOALLOC_MAX_PARTIALS];
@@ -32,39 +34,62 @@ __device__ __forceinline__ int ring_slot(long long t, int L) {
     return (int)(r < 0 ? r + L : r);
 }
 
-// Work item = (receiver tile, chunk of kernel steps); lane = receiver, warps split the steps.
-__global__ void __launch_bounds__(kThreads) noalloc_partial_kernel(const double* __restrict__ K, int n, int kmax,
+// The kernel tensor is kmax n rows (k, j) of n receivers, each read once: a stream, as long as enough of
+// it is in flight (134 MB at n = W = 256: 20 us at the copy rate; the 1.7e7 FP64 multiply-adds take 27 us at
+// two a clock and SM).  Work item = (receiver tile, range of rows); lane = receiver, the warps take
+// contiguous parts of the range, eight rows in flight each.  The ranges are as many as fill the GPU
+// (kFill CTAs), where the partial sums have room.  One item per 64 kernel steps, as before, left most
+// of the GPU idle: 1000 us at n = W = 256.
+__global__ void __launch_bounds__(kThreads) noalloc_partial_kernel(const double* __restrict__ K, int n, long long rows,
                                                                    const double* __restrict__ D, int hist_len,
-                                                                   int step, int nchunks, double* partial) {
-    __shared__ double red[kThreads / 32][32];
-    const int tile = blockIdx.x / nchunks, chunk = blockIdx.x % nchunks;
+                                                                   int step, int nsplit, double* partial) {
+    __shared__ double red[kWarps][kTile];
+    const int tile = blockIdx.x / nsplit, part = blockIdx.x % nsplit;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = tile * kTile + lane;
-    const int k0 = chunk * kSteps, k1 = min(kmax, k0 + kSteps);
-    double acc = 0.0;
-    for (int k = k0 + warp; k < k1; k += kThreads / 32) {
+    const long long w = (long long)part * kWarps + warp, nw = (long long)nsplit * kWarps;
+    const long long r0 = rows * w / nw, r1 = rows * (w + 1) / nw;
+    const double* Ki = K + (i < n ? i : n - 1);   // lanes past n read the last receiver, unused
+    double s0 = 0.0, s1 = 0.0;
+    long long k = r0 / n;
+    int j = (int)(r0 - k * n);
+    for (long long r = r0; r < r1; ++k, j = 0) {
         const double* Dk = D + (size_t)ring_slot((long long)step - k, hist_len) * n;
-        const double* Kk = K + (size_t)k * n * n;
-        if (i < n)
-            for (int j = 0; j < n; ++j) acc += Kk[(size_t)j * n + i] * Dk[j];
+        const long long e = min(r1, (k + 1) * n);   // the rows of kernel step k
+        for (; r + 8 <= e; r += 8, j += 8) {
+            double x[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[q] = __ldcs(Ki + (size_t)(r + q) * n);
+#pragma unroll
+            for (int q = 0; q < 8; q += 2) {
+                s0 = fma(x[q], Dk[j + q], s0);
+                s1 = fma(x[q + 1], Dk[j + q + 1], s1);
+            }
+        }
+        for (; r < e; ++r, ++j) s0 = fma(__ldcs(Ki + (size_t)r * n), Dk[j], s0);
     }
-    red[warp][lane] = acc;
+    red[warp][lane] = s0 + s1;
     __syncthreads();
     if (warp == 0) {
         double s = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) s += red[w][lane];
+        for (int q = 0; q < kWarps; ++q) s += red[q][lane];
         partial[(size_t)blockIdx.x * kTile + lane] = s;   // every slot of the item is written
     }
 }
 
-__global__ void noalloc_reduce_kernel(const double* partial, int n, int nchunks, double* T) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// one warp per receiver
+__global__ void noalloc_reduce_kernel(const double* partial, int n, int nsplit, double* T) {
+    const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    cudaGridDependencySynchronize();   // the partial sums are complete
     if (i >= n) return;
-    const int tile = i / kTile, lane = i % kTile;
+    const int tile = i / kTile, q = i % kTile;
     double s = 0.0;
-    for (int c = 0; c < nchunks; ++c) s += partial[((size_t)tile * nchunks + c) * kTile + lane];
-    T[i] = s;
+    for (int c = lane; c < nsplit; c += 32) s += partial[((size_t)tile * nsplit + c) * kTile + q];
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) T[i] = s;
 }
+
+const int kFill = 152 * 4;   // CTAs that fill the GPU
 
 }  // namespace
 
@@ -109,10 +134,24 @@ extern "C" int fdph_plain_step_noalloc(const double* K, int32_t n, int32_t W, co
         partial = g_addr[dev];
     }
     cudaStream_t s = (cudaStream_t)stream;
-    noalloc_partial_kernel<<<(unsigned)(tiles * nchunks), kThreads, 0, s>>>(K, n, kmax, D_hist, hist_len, step,
-                                                                             (int)nchunks, partial);
-    noalloc_reduce_kernel<<<(unsigned)(((long long)n + 127) / 128), 128, 0, s>>>(partial, n, (int)nchunks, T);
-    cudaError_t e = cudaGetLastError();
+    // parts of the rows: enough to fill the GPU, at least 8 rows a warp, no more than the array holds
+    const long long rows = (long long)kmax * n;
+    long long nsplit = std::min((kFill + tiles - 1) / tiles, rows / (8 * kWarps));
+    nsplit = std::max(1LL, std::min(nsplit, FDPH_NOALLOC_MAX_PARTIALS / (tiles * kTile)));
+    noalloc_partial_kernel<<<(unsigned)(tiles * nsplit), kThreads, 0, s>>>(K, n, rows, D_hist, hist_len, step, (int)nsplit,
+                                                                           partial);
+    // the reduction is launched while the sums are under way (it waits for them on the device)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(((long long)n * 32 + kThreads - 1) / kThreads));
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, noalloc_reduce_kernel, (const double*)partial, (int)n, (int)nsplit, T);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         fdph::set_error(std::string("fdph_plain_step_noalloc launch: ") + cudaGetErrorString(e));
         return FDPH_E_CUDA;
