@@ -90,21 +90,33 @@ __global__ void __launch_bounds__(32 * kTcWarps, 3) tc_block_kernel(StepArgs<flo
     __half* rows = (__half*)tc_smem;
     float* scl = (float*)(tc_smem + Cf::row_bytes(nk > 0 ? nk : 1));
     {
-        const int top = n + B - 1 - tk.k0, hend = hist_end(a, n);
+        const int top = n + B - 1 - tk.k0, hend = hist_end(a, n), stop = wrap(top, a.WD);
         const float* ring = a.Dring32 + tk.s0 + (lane < ns ? lane : 0);
-#pragma unroll 4
-        for (int u = warp; u < nrow * NR; u += kTcWarps) {
-            const int q = u / NR, r = u - q * NR, t = top - q;
-            const bool ok = t >= 0 && t < hend;
-            const int slot = wrap(t, a.WD);
-            const float x = ok && lane < ns ? ring[r * a.rs_D + (size_t)slot * a.N] : 0.f;
-            const float sc = ok ? a.Dscale[(size_t)slot * NR + r] : 0.f;
-            // 2^sh from 2^-sh: the exponents add up to that of 1
-            const float y = x * (ok ? __uint_as_float((254u << 23) - __float_as_uint(sc)) : 0.f);
-            const __half hi = __float2half_rn(y);
-            rows[(size_t)(q * C + r) * 32 + lane] = hi;
-            rows[(size_t)(q * C + NR + r) * 32 + lane] = __float2half_rn(y - __half2float(hi));
-            if (lane == 0) scl[q * C + r] = scl[q * C + NR + r] = sc;
+        // (the loads of kAhead rows in flight at a time: a row is a dependent pair of loads otherwise, and
+        // the staging, not the MMAs, bounded the kernel)
+        constexpr int kAhead = 8;
+        for (int u0 = warp * kAhead; u0 < nrow * NR; u0 += kTcWarps * kAhead) {
+            float x[kAhead], sc[kAhead];
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) {
+                const int u = u0 + i, q = u / NR, r = u % NR, t = top - q;
+                const bool ok = u < nrow * NR && t >= 0 && t < hend;
+                int slot = stop - q;              // nrow <= WD: one wrap at most
+                slot += slot < 0 ? a.WD : 0;
+                x[i] = ok && lane < ns ? ring[r * a.rs_D + (size_t)slot * a.N] : 0.f;
+                sc[i] = ok ? a.Dscale[(size_t)slot * NR + r] : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) {
+                const int u = u0 + i, q = u / NR, r = u % NR;
+                if (u >= nrow * NR) break;
+                // 2^sh from 2^-sh: the exponents add up to that of 1
+                const float y = x[i] * (sc[i] > 0.f ? __uint_as_float((254u << 23) - __float_as_uint(sc[i])) : 0.f);
+                const __half hi = __float2half_rn(y);
+                rows[(size_t)(q * C + r) * 32 + lane] = hi;
+                rows[(size_t)(q * C + NR + r) * 32 + lane] = __float2half_rn(y - __half2float(hi));
+                if (lane == 0) scl[q * C + r] = scl[q * C + NR + r] = sc[i];
+            }
         }
     }
     __syncthreads();
