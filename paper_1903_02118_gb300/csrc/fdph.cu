@@ -688,7 +688,16 @@ static void enqueue_rupture_h(fdph_plan_t P, StepArgs<T> a, double* D, cudaStrea
     a.T_out = T_out;
     for (int b = 0; b < a.nb; ++b) {
         ProfScope ps(P, 0, 1);
-        rup_step_kernel<T, H><<<a.n_groups, kRupThreads, 0, s>>>(a, P->fr, D, b, recent);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(a.n_groups);
+        cfg.blockDim = dim3(kRupThreads);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = b > 0 && !P->prof ? 1 : 0;   // (a step's launch overlaps the step before)
+        cudaLaunchKernelEx(&cfg, rup_step_kernel<T, H>, a, P->fr, D, b, recent);
     }
     if (a.n_fir) { ProfScope ps(P, 1, a.nb); launch_fir<T>(a, s); }
     { ProfScope ps(P, 2, a.nb); launch_eq42<T>(a, s); }
@@ -1267,7 +1276,7 @@ static int build_recent(fdph_plan_t P) {
         groups[g].nleaf = (int)per[g].size();
         for (int l : per[g]) {
             const NearLeaf& L = hp.near[l];
-            leaves.push_back({(long long)L.tensor, L.sl, L.r0, L.nr, L.s0, L.ns, L.kz, L.W, 0});
+            leaves.push_back({(long long)L.tensor, L.sl, L.r0, L.nr, L.s0, L.ns, L.kz, L.W, {0, 0, 0}});
         }
     }
     P->n_groups = (int)groups.size();

@@ -90,8 +90,9 @@ struct RecGroup {
 };
 struct __align__(16) RecLeaf {
     long long off;       // element offset of kernel step 0
-    int sl, r0, nr, s0, ns, kz, W, pad;
+    int sl, r0, nr, s0, ns, kz, W, pad[3];
 };
+static_assert(sizeof(RecLeaf) == 48, "a leaf is three 16-byte loads");
 
 static const int kMaxSoe = 16;
 static const int kMaxRhs = 8;    // right-hand sides of one plan at most (1, 2, 4 or 8)
@@ -936,78 +937,144 @@ struct FrictionDev {
 // steps 1 ... n - n0 of the near leaves that a wave crosses that fast (RecLeaf: the first kz kernel
 // steps of a leaf vanish; the far blocks and the static and tail terms act later than kBlk steps, see
 // rup_block).  One CTA per receiver group (the disjoint maximal receiver clusters of those leaves): its
-// warps take the (leaf, kernel step) pairs in turn, then the first warp solves the friction law and
+// warps take the (leaf, kernel step) units in turn, then the first warp solves the friction law and
 // appends the slip rate (push).  b: the step within the launch sequence's block.
+//
+// The steps of a block follow one another, so the kernel's latency bounds a rupture.  It is launched
+// while the step before is still running (programmatic dependent launch): what does not depend on that
+// step (unit lists, the first unit's coefficients, prestress and history traction) is loaded before
+// the wait.
 static const int kRupThreads = 512;
+static const int kRupLeaves = 32;    // leaves of a group kept in shared memory
 
 template <class T, class H>
-__global__ void __launch_bounds__(kRupThreads) rup_step_kernel(StepArgs<T> a, FrictionDev f, double* D, int b, int recent) {
+__global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_kernel(StepArgs<T> a, FrictionDev f, double* D, int b, int recent) {
     using R = typename NearTypes<H>::Row;
     constexpr int V = 16 / (int)sizeof(H), W = kRupThreads / 32;
-    __shared__ __align__(16) R row[W][36];
+    constexpr int NB = 32 / V;                            // 16-byte vectors of a slice per receiver
+    __shared__ __align__(16) R row[W][2][36];
     __shared__ double red[W][32];
+    __shared__ RecLeaf leaves[kRupLeaves];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const RecGroup g = a.rec_groups[blockIdx.x];
     const int nf = step_index(a), n = nf + b;
     const int back = recent ? n - (n & ~(kBlk - 1)) : 0;   // the block's earlier steps
     red[warp][lane] = 0.0;
-    int unit = 0;
-    for (int q = 0; q < g.nleaf; ++q) {
-        const RecLeaf L = a.rec_leaves[g.leaf0 + q];
-        const int k0 = max(L.kz, 1), k1 = min(back + 1, L.W);
-        const int nbk = (L.ns + V - 1) / V;
-        // this warp's kernel steps of the leaf: those whose running number is its own modulo W
-        int k = k0 + ((warp - unit) % W + W) % W;
-        unit += max(k1 - k0, 0);
-        for (; k < k1; k += W) {
-            const size_t off = (size_t)wrap(n - k, a.WD) * a.N + L.s0 + min(lane, L.ns - 1);
-            R v;
-            if constexpr (sizeof(R) == 4) v = a.Dring32[off]; else v = a.Dring[off];
-            const H* sl = (const H*)a.tensor + L.off + (size_t)k * L.sl + (size_t)(lane < L.nr ? lane : 0) * V;
-            const bool in = FDPH_IDX(L.off + (long long)(k + 1) * L.sl <= a.len_tensor, a.err);
-            __syncwarp();
-            row[warp][lane] = lane < L.ns ? v : (R)0;
-            __syncwarp();
-            R s = 0;
-#pragma unroll 8
-            for (int jb = 0; jb < nbk; ++jb) {
-                const uint4 u = in ? *(const uint4*)(sl + (size_t)jb * L.nr * V) : make_uint4(0, 0, 0, 0);
-                R x[V], y[V];
-                if constexpr (sizeof(H) == 2) unpack(u, x, __half());
-                else unpack(u, x, R());
-                load_row<V>(&row[warp][jb * V], y);
-                R t = x[0] * y[0];
-#pragma unroll
-                for (int q2 = 1; q2 < V; ++q2) t = fma(x[q2], y[q2], t);
-                s += t;
-            }
-            if (lane < L.nr && FDPH_IDX(L.r0 - g.r0 >= 0 && L.r0 - g.r0 + L.nr <= 32, a.err))
-                red[warp][L.r0 - g.r0 + lane] += (double)s * (double)a.kinv;
-            __syncwarp();
-        }
+    {
+        constexpr int words = (int)(sizeof(RecLeaf) / 16);
+        const int m = min(g.nleaf, kRupLeaves) * words;
+        for (int q = threadIdx.x; q < m; q += kRupThreads) ((int4*)leaves)[q] = ((const int4*)(a.rec_leaves + g.leaf0))[q];
+    }
+    // the first warp's element
+    const bool mine = warp == 0 && lane < g.nr;
+    const int p = g.r0 + lane, e = mine ? a.perm[p] : 0;
+    double T0 = 0.0, tau0 = 0.0, k0 = -1.0;
+    if (mine) {
+        T0 = a.thist[(size_t)b * a.N + p];
+        tau0 = f.tau0[e];
+        k0 = f.k0[e];
     }
     __syncthreads();
-    if (warp || lane >= g.nr) return;
-    const int p = g.r0 + lane, e = a.perm[p];
-    double T0 = a.thist[(size_t)b * a.N + p];
-    for (int w = 0; w < W; ++w) T0 += red[w][lane];
+    auto leaf = [&](int q) -> RecLeaf { return q < kRupLeaves ? leaves[q] : a.rec_leaves[g.leaf0 + q]; };
+    auto range = [&](const RecLeaf& L, int& first) {
+        first = max(L.kz, 1);
+        return max(min(back + 1, L.W) - first, 0);   // kernel steps first, first + 1, ...
+    };
+    // the unit with running number r from leaf q on: its leaf (nleaf: none) and kernel step
+    auto seek = [&](int& q, int r, RecLeaf& L, int& k) {
+        for (; q < g.nleaf; ++q) {
+            int first;
+            L = leaf(q);
+            const int len = range(L, first);
+            if (r < len) {
+                k = first + r;
+                return;
+            }
+            r -= len;
+        }
+    };
+    auto load_x = [&](const RecLeaf& L, int k, uint4 (&x)[NB]) {
+        const H* sl = (const H*)a.tensor + L.off + (size_t)k * L.sl + (size_t)(lane < L.nr ? lane : 0) * V;
+        const bool in = FDPH_IDX(L.off + (long long)(k + 1) * L.sl <= a.len_tensor, a.err);
+#pragma unroll
+        for (int jb = 0; jb < NB; ++jb)
+            x[jb] = in && jb * V < L.ns ? *(const uint4*)(sl + (size_t)jb * L.nr * V) : make_uint4(0, 0, 0, 0);
+    };
+    auto load_v = [&](const RecLeaf& L, int k) -> R {
+        const size_t off = (size_t)wrap(n - k, a.WD) * a.N + L.s0 + min(lane, L.ns - 1);
+        R v;
+        if constexpr (sizeof(R) == 4) v = a.Dring32[off]; else v = a.Dring[off];
+        return lane < L.ns ? v : (R)0;
+    };
+    RecLeaf L;
+    int q = 0, k = 0;
+    uint4 x[NB];
+    seek(q, warp, L, k);
+    if (q < g.nleaf) load_x(L, k, x);
+    cudaGridDependencySynchronize();                 // the step before is complete
+    cudaTriggerProgrammaticLaunchCompletion();
+    double u = 0.0, c = 0.0, comp = 0.0;
+    if (mine) {
+        u = f.slip[e];
+        c = a.C[p];
+        comp = a.Ccomp[p];
+    }
+    R v = q < g.nleaf ? load_v(L, k) : (R)0;
+    for (int buf = 0; q < g.nleaf; buf ^= 1) {
+        row[warp][buf][lane] = v;
+        __syncwarp();
+        const int ns = L.ns, nr = L.nr, r0 = L.r0 - g.r0;
+        // the unit W further: its slip rates are loaded meanwhile, its coefficients next
+        {
+            int first;
+            range(L, first);
+            seek(q, k - first + W, L, k);
+        }
+        if (q < g.nleaf) v = load_v(L, k);
+        R s = 0;
+#pragma unroll
+        for (int jb = 0; jb < NB; ++jb) {
+            if (jb * V >= ns) break;
+            R xv[V], y[V];
+            if constexpr (sizeof(H) == 2) unpack(x[jb], xv, __half());
+            else unpack(x[jb], xv, R());
+            load_row<V>(&row[warp][buf][jb * V], y);
+            R t = xv[0] * y[0];
+#pragma unroll
+            for (int i = 1; i < V; ++i) t = fma(xv[i], y[i], t);
+            s += t;
+        }
+        if (q < g.nleaf) load_x(L, k, x);
+        if (lane < nr && FDPH_IDX(r0 >= 0 && r0 + nr <= 32, a.err)) red[warp][r0 + lane] += (double)s * (double)a.kinv;
+        __syncwarp();
+    }
+    __syncthreads();
+    if (!mine) return;
+    {
+        double t[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) t[w] = red[w][lane];
+#pragma unroll
+        for (int h = W / 2; h; h >>= 1)
+#pragma unroll
+            for (int w = 0; w < h; ++w) t[w] += t[w + h];
+        T0 += t[0];
+    }
     const long long off = io_offset(a, nf) + (long long)b * a.io_stride + e;
-    const double tau = f.tau0[e] + T0;
-    const double u = f.slip[e];
+    const double tau = tau0 + T0;
     double strength;
     if (f.law == 1) {
         strength = f.sigma_n * (f.mu_d + (f.mu_s - f.mu_d) * exp(-u / f.Dc));
     } else {
-        const double x = u < f.Dc ? u / f.Dc : 1.0;
-        strength = f.sigma_n * (f.mu_s - (f.mu_s - f.mu_d) * x);
+        const double w = u < f.Dc ? u / f.Dc : 1.0;
+        strength = f.sigma_n * (f.mu_s - (f.mu_s - f.mu_d) * w);
     }
-    const double eta = -f.k0[e];
-    const double v = tau > strength ? (tau - strength) / eta : 0.0;
-    D[off] = v;
-    a.T_out[off] = tau + f.k0[e] * v;
-    f.slip[e] = u + v * f.dt;
-    double c = a.C[p], comp = a.Ccomp[p];
-    push_one(a, p, n, b, v, c, comp);
+    const double eta = -k0;
+    const double d = tau > strength ? (tau - strength) / eta : 0.0;
+    push_one(a, p, n, b, d, c, comp);
+    D[off] = d;
+    a.T_out[off] = tau + k0 * d;
+    f.slip[e] = u + d * f.dt;
     a.C[p] = c;
     a.Ccomp[p] = comp;
 }
