@@ -47,6 +47,7 @@
 #include "../../include/fdph.h"
 #include "internal.h"
 #include "kernel2d.cuh"
+#include "fixed.cuh"
 #include "plan.h"
 #include "step.cuh"
 #include "tensor.cuh"
@@ -297,6 +298,9 @@ struct fdph_plan_s {
     int n_win = 0, n_aux = 0; // window and aux items (tensor cores: the window items first)
     void* tensor = nullptr;
     void* stat = nullptr;     // aux slices, storage type
+    int *fx_win = nullptr, *fx_aux = nullptr;   // FP64: slice exponents (fixed.cuh)
+    double* rec_tensor = nullptr;               // FP64: the rupture leaves' first kBlk kernel steps as numbers
+    long long rec_len = 0;
     int *np_ptr = nullptr, *np_idx = nullptr;
     int* err = nullptr;
     double* rho = nullptr;
@@ -468,6 +472,10 @@ static StepArgs<T> make_args(fdph_plan_t P, const double* D, double* T_) {
     a.n_items = P->n_win + P->n_aux;
     a.tensor = P->tensor;
     a.kinv = (float)(1.0 / P->kscale);
+    a.fx_win = P->fx_win;
+    a.fx_aux = P->fx_aux;
+    a.rec_tensor = P->rec_tensor ? P->rec_tensor : P->tensor;
+    a.len_rec = P->rec_tensor ? P->rec_len : hp.near_tensor_len;
     a.stat = P->stat;
     a.len_tensor = hp.near_tensor_len;
     a.len_aux = hp.near_aux_len;
@@ -573,6 +581,13 @@ static void launch_tc(StepArgs<float> a, int n_win, int chunk, cudaStream_t s) {
 
 template <class T, class H>
 static void launch_near_h(fdph_plan_t P, StepArgs<T> a, cudaStream_t s) {
+    if constexpr (sizeof(H) == 8) {   // FP64: exact products on the tensor cores
+        if (!a.n_items) return;
+        const dim3 g(a.n_items, a.nrhs);
+        if (a.nb == 1) fixed_block_kernel<1><<<g, 32 * kFxWarps, FxCfg<1>::smem(P->chunk), s>>>(a, P->chunk);
+        else fixed_block_kernel<kBlk><<<g, 32 * kFxWarps, FxCfg<kBlk>::smem(P->chunk), s>>>(a, P->chunk);
+        return;
+    } else {
     if constexpr (std::is_same<H, __half>::value) {
         if (P->nrhs >= 2) {
             if (P->n_win) {
@@ -587,6 +602,7 @@ static void launch_near_h(fdph_plan_t P, StepArgs<T> a, cudaStream_t s) {
     if (!a.n_items) return;
     if (a.nb == 1) launch_near_items<T, H, 1>(a, P->chunk, s);
     else launch_near_items<T, H, kBlk>(a, P->chunk, s);
+    }
 }
 
 template <class T>
@@ -939,6 +955,16 @@ static int launch_commit(fdph_plan_t P, const double* D_n) {
     return FDPH_OK;
 }
 
+// first slice of every leaf among the plan's window and aux slices
+static void slice_numbers(const HostPlan& hp, std::vector<long long>& win0, std::vector<long long>& aux0) {
+    win0.assign(1, 0);
+    aux0.assign(1, 0);
+    for (const NearLeaf& L : hp.near) {
+        win0.push_back(win0.back() + L.W);
+        aux0.push_back(aux0.back() + L.naux);
+    }
+}
+
 // The plan's near-field work items as the near kernels read them: window items first where they go to
 // the tensor cores, else all together, largest first (an item is a warp's or a CTA's work: the last to
 // start are the shortest).
@@ -950,6 +976,8 @@ static int build_schedule(fdph_plan_t P) {
     const int ni = (int)hp.items.size();
     std::vector<NearTask> all(ni);
     std::vector<double> cost(ni);
+    std::vector<long long> win0, aux0;
+    slice_numbers(hp, win0, aux0);
     P->n_win = P->n_aux = 0;
     for (int q = 0; q < ni; ++q) {
         const NearItem& it = hp.items[q];
@@ -967,6 +995,7 @@ static int build_schedule(fdph_plan_t P) {
         t.s0 = L.s0;
         t.W = L.W;
         t.vstate = (int)L.vstate;
+        t.slice = it.k0 + (int)(it.kind ? aux0[it.leaf] : win0[it.leaf]);
         // bytes, and for aux slices the FP64 work of their rows and sums
         cost[q] = (double)(it.k1 - it.k0) * (t.sl * (double)(it.kind ? sizeof(A) : sizeof(H)) + (it.kind ? 4096.0 : 0.0)) + 4096.0;
         (it.kind ? P->n_aux : P->n_win) += 1;
@@ -988,10 +1017,15 @@ static int build_schedule(fdph_plan_t P) {
         FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8, 1>::smem(kChunk)));
         FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8, 8>::smem(kChunk)));
     }
-    FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, H, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)NearCfg<H, 1>::warp_bytes(2 * kChunk) * kNearWarps));
-    FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, H, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)NearCfg<H, kBlk>::warp_bytes(2 * kChunk) * kNearWarps));
+    if constexpr (sizeof(H) == 8) {
+        FDPH_CUDA(cudaFuncSetAttribute(fixed_block_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FxCfg<1>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(fixed_block_kernel<kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FxCfg<kBlk>::smem(kChunk)));
+    } else {
+        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, H, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)NearCfg<H, 1>::warp_bytes(2 * kChunk) * kNearWarps));
+        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, H, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)NearCfg<H, kBlk>::warp_bytes(2 * kChunk) * kNearWarps));
+    }
     P->sched_version += 1;
     int rc;
     if ((rc = upload(P, &P->tasks, tasks)) || (rc = upload(P, &P->np_ptr, hp.np_ptr)) || (rc = upload(P, &P->np_idx, hp.np_idx)))
@@ -1232,6 +1266,32 @@ static int build_near_finish(fdph_plan_t P, const PlanInputs& in, NearBuild& nb)
                                       cudaMemcpyHostToDevice, P->stream));
     }
     stamp("near: tail fits");
+    if constexpr (sizeof(H) == 8) {
+        // the rupture leaves' first kernel steps stay as numbers; then all slices take the form of fixed.cuh
+        for (const NearLeaf& L : hp.near)
+            if (L.kz < kBlk) P->rec_len += (long long)std::min(L.W, kBlk) * L.sl;
+        if ((rc = dalloc(P, &P->rec_tensor, (size_t)P->rec_len))) return rc;
+        long long at = 0;
+        for (const NearLeaf& L : hp.near)
+            if (L.kz < kBlk) {
+                const size_t c = (size_t)std::min(L.W, kBlk) * L.sl;
+                if (c) FDPH_CUDA(cudaMemcpyAsync(P->rec_tensor + at, (const double*)P->tensor + L.tensor, c * sizeof(double),
+                                                 cudaMemcpyDeviceToDevice, P->stream));
+                at += (long long)c;
+            }
+        std::vector<long long> win0, aux0;
+        slice_numbers(hp, win0, aux0);
+        long long *d_win0 = nullptr, *d_aux0 = nullptr;
+        if ((rc = upload(P, &d_win0, win0)) || (rc = upload(P, &d_aux0, aux0)) || (rc = dalloc(P, &P->fx_win, (size_t)win0.back() * 2)) ||
+            (rc = dalloc(P, &P->fx_aux, (size_t)aux0.back() * 2)))
+            return rc;
+        const int nl = (int)hp.near.size();
+        if (nl) {
+            fx_pack_kernel<<<nl, 256, 0, P->stream>>>((double*)P->tensor, P->fx_win, P->near, d_win0, 0, hp.soe);
+            fx_pack_kernel<<<nl, 256, 0, P->stream>>>((double*)P->stat, P->fx_aux, P->near, d_aux0, 1, hp.soe);
+            FDPH_CUDA(cudaGetLastError());
+        }
+    }
     if ((rc = build_schedule<T, H>(P))) return rc;
     FDPH_CUDA(cudaStreamSynchronize(P->stream));
     return FDPH_OK;
@@ -1271,12 +1331,20 @@ static int build_recent(fdph_plan_t P) {
     std::vector<RecLeaf> leaves;
     std::vector<std::vector<int>> per(groups.size());
     for (int l : use) per[group_of[hp.near[l].r0]].push_back(l);
+    std::vector<long long> at(hp.near.size(), 0);   // FP64: place in rec_tensor
+    if (P->rec_tensor) {
+        long long o = 0;
+        for (int l : use) {
+            at[l] = o;
+            o += (long long)std::min(hp.near[l].W, kBlk) * hp.near[l].sl;
+        }
+    }
     for (size_t g = 0; g < groups.size(); ++g) {
         groups[g].leaf0 = (int)leaves.size();
         groups[g].nleaf = (int)per[g].size();
         for (int l : per[g]) {
             const NearLeaf& L = hp.near[l];
-            leaves.push_back({(long long)L.tensor, L.sl, L.r0, L.nr, L.s0, L.ns, L.kz, L.W, {0, 0, 0}});
+            leaves.push_back({P->rec_tensor ? at[l] : (long long)L.tensor, L.sl, L.r0, L.nr, L.s0, L.ns, L.kz, L.W, {0, 0, 0}});
         }
     }
     P->n_groups = (int)groups.size();
@@ -1357,7 +1425,7 @@ static void fill_stats(fdph_plan_t P) {
     s.state_bytes = (long long)P->state_bytes;
     long long arena = 0;
     arena += (long long)(hp.fac.size() * ps) + hp.ints.size() * 4 + hp.sbs.size() * sizeof(SbDev);
-    arena += (long long)(hp.near_tensor_len * pw + hp.near_aux_len * ps);
+    arena += (long long)(hp.near_tensor_len * pw + hp.near_aux_len * ps) + P->rec_len * 8;
     s.arena_bytes = arena;
 }
 

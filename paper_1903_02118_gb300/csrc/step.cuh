@@ -63,7 +63,8 @@ struct NearDev {
 struct __align__(16) NearTask {
     long long off;       // element offset of the item's first slice (tensor, or aux for kind 1)
     int item, k0, k1, kind, nr, ns, sl, s0, W, vstate;
-    int pad[2];
+    int slice;           // FP64 plans: number of the item's first slice among the plan's slices of its kind
+    int pad;
 };
 static_assert(sizeof(NearTask) == 64, "one work item is four 16-byte loads");
 
@@ -151,8 +152,11 @@ struct StepArgs {
     int n_items;
     const void* tensor;       // near-field window slices (window storage type)
     float kinv;               // inverse of the window coefficients' storage scale (FP16: 2^-e, else 1)
+    const int *fx_win, *fx_aux;   // FP64 plans: exponents of the slices (fixed.cuh), [slice][2]
+    const void* rec_tensor;   // the kernel steps of a rupture block's own part (RecLeaf::off), window storage
+                              // type (FP64 plans: as numbers, not in the form of fixed.cuh)
     const void* stat;         // aux slices: static tiles, exponential-tail coefficients (aux storage type)
-    long long len_tensor, len_aux;   // elements of tensor and stat (index checks of FDPH_CHECK builds)
+    long long len_tensor, len_aux, len_rec;   // elements of tensor, stat and rec_tensor (index checks of FDPH_CHECK builds)
     double* partial;          // [kBlk][cap_partial]: [item][32] per step
     long long cap_partial;
     const int* np_ptr;
@@ -228,6 +232,32 @@ __device__ __forceinline__ StepArgs<T> rhs_args(const StepArgs<T>& a0, int r) {
         if (a0.uhist) a.uhist = a0.uhist + r * a0.len_uhist;
     }
     return a;
+}
+
+// Conversions between FP32 and FP64 in integer arithmetic.  The hardware's run on the FP64 pipe, two
+// lanes a clock and SM like its additions (a warp takes 15 clocks; the integer forms take 3 to 6), and
+// the FP64 pipe bounds the far field and the aux slices.  Same values: exact widening, narrowing to
+// nearest even; zeros here, subnormals, infinities and NaN by the hardware conversion.
+__device__ __forceinline__ double wide(double x) { return x; }
+__device__ __forceinline__ double wide(float x) {
+    const unsigned u = __float_as_uint(x);
+    if (((u >> 23) & 0xffu) - 1u < 254u)
+        return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+    if (!(u << 1)) return __hiloint2double((int)u, 0);
+    return (double)x;
+}
+__device__ __forceinline__ double narrow(double x, double) { return x; }
+__device__ __forceinline__ float narrow(double x, float) {
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+    const unsigned e = (h >> 20) & 0x7ffu;
+    if (e - 897u <= 253u) {   // a normal FP32 number (or rounded up to infinity)
+        unsigned v = (((h & 0x7fffffffu) - 0x38000000u) << 3) | (l >> 29);
+        const unsigned rem = l & 0x1fffffffu;
+        v += rem > 0x10000000u || (rem == 0x10000000u && (v & 1u)) ? 1u : 0u;
+        return __uint_as_float((h & 0x80000000u) | v);
+    }
+    if (!((h << 1) | l)) return __uint_as_float(h);
+    return (float)x;
 }
 
 __global__ void advance_step_kernel(int* n_dev, int k) { *n_dev += k; }
@@ -360,13 +390,17 @@ __global__ void __launch_bounds__(32 * kFirWarps) fir_kernel(StepArgs<T> a0, boo
             T x[2 * B - 1];
 #pragma unroll
             for (int q = 0; q < 2 * B - 1; ++q) x[q] = d_at(min(m0 + q, rows + B - 1));
+            constexpr int F = sizeof(T) == 4 ? B : B / 4;   // taps in flight together (registers)
 #pragma unroll
-            for (int u = 0; u < B; ++u) {
-                if (m0 + u >= g.taps) break;
-                const T hm = h[(size_t)(m0 + u) * 32];
+            for (int v = 0; v < B; v += F) {
+                T hm[F];
 #pragma unroll
-                for (int b = 0; b < B; ++b)
-                    (u & 1 ? s1 : s0)[b] = fma(hm, x[B - 1 - b + u], (u & 1 ? s1 : s0)[b]);
+                for (int u = 0; u < F; ++u) hm[u] = m0 + v + u < g.taps ? h[(size_t)(m0 + v + u) * 32] : (T)0;
+#pragma unroll
+                for (int u = 0; u < F; ++u)
+#pragma unroll
+                    for (int b = 0; b < B; ++b)
+                        (u & 1 ? s1 : s0)[b] = fma(hm[u], x[B - 1 - b + v + u], (u & 1 ? s1 : s0)[b]);
             }
         }
     }
@@ -385,7 +419,7 @@ __global__ void __launch_bounds__(32 * kFirWarps) fir_kernel(StepArgs<T> a0, boo
 // (Domain S, App. B.1), slip rate (transient)
 template <class T>
 __device__ __forceinline__ double source_value(const StepArgs<T>& a, const SbDev& sb, int jl, int b) {
-    if (sb.kind == 0) return (double)a.dhat[(sb.dhat + jl) * kBlk + b];
+    if (sb.kind == 0) return wide(a.dhat[(sb.dhat + jl) * kBlk + b]);
     return (sb.kind == 1 ? a.blkC : a.blkD)[(size_t)(sb.s0 + jl) * kBlk + b];
 }
 
@@ -434,12 +468,12 @@ __global__ void scatter_kernel(StepArgs<T> a0) {
             const int b = d - rn.x;
             if (b >= nb) break;
             if (rn.y == 1) {
-                v = fma((double)g[(long long)rn.w * rank + l], source_value(a, sb, rn.w, b), v);
+                v = fma(wide(g[(long long)rn.w * rank + l]), source_value(a, sb, rn.w, b), v);
             } else {
                 double s = 0.0;
                 for (int u = 0; u < rn.y; ++u) {
                     const int jl = a.src_order[rn.z + u];
-                    s = fma((double)g[(long long)jl * rank + l], source_value(a, sb, jl, b), s);
+                    s = fma(wide(g[(long long)jl * rank + l]), source_value(a, sb, jl, b), s);
                 }
                 v += s;
             }
@@ -541,7 +575,7 @@ __global__ void __launch_bounds__(32 * kTrWarps) trconv_kernel(StepArgs<T> a0) {
             }
             __syncwarp();
             if (m0 + lane < sb.taps) {
-                const double hm = (double)a.fac[sb.h + m0 + lane];
+                const double hm = wide(a.fac[sb.h + m0 + lane]);
 #pragma unroll
                 for (int b = 0; b < B; ++b) z[b] = fma(hm, ys[warp][B - 1 - b + lane], z[b]);
             }
@@ -593,7 +627,7 @@ __global__ void __launch_bounds__(128) far_kernel(StepArgs<T> a0) {
         const bool id = en.flags & 2;
         const int l0 = id ? (int)en.f : 0, l1 = id ? l0 + 1 : en.rank;
         for (int l = l0; l < l1; ++l) {
-            const double f = id ? 1.0 : (double)a.fac[en.f + l];
+            const double f = id ? 1.0 : wide(a.fac[en.f + l]);
 #pragma unroll
             for (int b = 0; b < B; ++b) {
                 int s = slot + b;   // L >= kBlk: one wrap at most
@@ -639,7 +673,7 @@ __global__ void gather_kernel(StepArgs<T> a0) {
     }
 }
 
-// ---- near field (App. E) on the CUDA cores
+// ---- near field (App. E) on the CUDA cores (FP32 and FP16 plans; FP64: fixed.cuh)
 
 // Near-field storage: window slices in H; aux slices (static tile, tail coefficients) in the aux
 // type (FP32 when the window is FP16: the static term multiplies the cumulative slip, so its
@@ -692,8 +726,8 @@ static const int kNearWarps = 4;   // work items (warps) of a near-field CTA
 template <class H, int B>
 struct NearCfg {
     using R = typename NearTypes<H>::Row;
-    static constexpr int G = sizeof(H) == 8 ? 2 : 4;                  // window slices taken together
-    static constexpr int pitch = sizeof(R) == 8 ? 34 : 36;            // row of 32 entries, padded
+    static constexpr int G = 4;                                       // window slices taken together
+    static constexpr int pitch = 36;                                  // row of 32 entries, padded
     // shared memory of one warp: the rows of a window item of `chunk` slices, or an aux item's
     // slip rates (FP64) and one row of B steps for each of its lane groups' slices
     static constexpr size_t warp_bytes(int chunk) {
@@ -790,21 +824,7 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
                     }
                     const bool wrapj = jb + 1 == nbk;
                     load(wrapj ? gr + ngrp : gr, wrapj ? 0 : jb + 1, xn);
-                    if constexpr (sizeof(R) == 8) {
-#pragma unroll
-                        for (int q = 0; q < B + G - 1; ++q) {
-                            R y[V];
-                            load_row<V>(rg + q * P + jb * V, y);
-#pragma unroll
-                            for (int g = 0; g < G; ++g) {
-                                const int b = B - 1 - q + g;
-                                if (b >= 0 && b < B) {
-#pragma unroll
-                                    for (int v = 0; v < V; ++v) acc[b] = fma(x[g][v], y[v], acc[b]);
-                                }
-                            }
-                        }
-                    } else {
+                    {
                         R s[B];
 #pragma unroll
                         for (int b = 0; b < B; ++b) s[b] = 0;
@@ -825,14 +845,12 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
                         for (int b = 0; b < B; ++b) ga[b] += s[b];
                     }
                 }
-                if constexpr (sizeof(R) == 4) {
 #pragma unroll
-                    for (int b = 0; b < B; ++b) acc[b] += ga[b];
-                }
+                for (int b = 0; b < B; ++b) acc[b] += ga[b];
             }
             // window sums carry the storage scale of the window (FP16)
 #pragma unroll
-            for (int b = 0; b < B; ++b) tot[b] = (double)acc[b] * (double)a.kinv;
+            for (int b = 0; b < B; ++b) tot[b] = wide(acc[b] * (R)a.kinv);   // (a power of two)
         }
     } else {
         // aux slices: slice 0 the static tile (times C_j(n - W), it carries dt), slice 1 + q the tail
@@ -870,14 +888,14 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
 #pragma unroll
                 for (int b = 0; b < B; ++b)
                     vr[b * (span + 4) + ri] =
-                        (R)(b < nb && src && t0 + b >= 0 ? Cr[(size_t)wrap(t0 + b, a.WC) * a.N] : 0.0);
+                        narrow(b < nb && src && t0 + b >= 0 ? Cr[(size_t)wrap(t0 + b, a.WC) * a.N] : 0.0, R());
             } else if (on) {
                 const double rho = a.rho[ai - 1];
                 double v = src ? vs[(size_t)(ai - 1) * ns] : 0.0;
 #pragma unroll
                 for (int b = 0; b < B; ++b) {
                     if (b < nb) v = fma(rho, v, dw[b * 32 + ri]);
-                    vr[b * (span + 4) + ri] = (R)(src && b < nb ? v : 0.0);
+                    vr[b * (span + 4) + ri] = narrow(src && b < nb ? v : 0.0, R());
                 }
                 if (src) vs[(size_t)(ai - 1) * ns] = v;
             }
@@ -903,7 +921,7 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
                 }
                 // FP64 across slices
 #pragma unroll
-                for (int b = 0; b < B; ++b) tot[b] += (double)t[b];
+                for (int b = 0; b < B; ++b) tot[b] += wide(t[b]);
             }
             __syncwarp();
         }
@@ -994,8 +1012,8 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
         }
     };
     auto load_x = [&](const RecLeaf& L, int k, uint4 (&x)[NB]) {
-        const H* sl = (const H*)a.tensor + L.off + (size_t)k * L.sl + (size_t)(lane < L.nr ? lane : 0) * V;
-        const bool in = FDPH_IDX(L.off + (long long)(k + 1) * L.sl <= a.len_tensor, a.err);
+        const H* sl = (const H*)a.rec_tensor + L.off + (size_t)k * L.sl + (size_t)(lane < L.nr ? lane : 0) * V;
+        const bool in = FDPH_IDX(L.off + (long long)(k + 1) * L.sl <= a.len_rec, a.err);
 #pragma unroll
         for (int jb = 0; jb < NB; ++jb)
             x[jb] = in && jb * V < L.ns ? *(const uint4*)(sl + (size_t)jb * L.nr * V) : make_uint4(0, 0, 0, 0);
@@ -1045,7 +1063,7 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
             s += t;
         }
         if (q < g.nleaf) load_x(L, k, x);
-        if (lane < nr && FDPH_IDX(r0 >= 0 && r0 + nr <= 32, a.err)) red[warp][r0 + lane] += (double)s * (double)a.kinv;
+        if (lane < nr && FDPH_IDX(r0 >= 0 && r0 + nr <= 32, a.err)) red[warp][r0 + lane] += wide(s * (R)a.kinv);
         __syncwarp();
     }
     __syncthreads();

@@ -192,12 +192,13 @@ __global__ void __launch_bounds__(32 * kTcWarps, 3) tc_block_kernel(StepArgs<flo
             }
     __syncthreads();
     if (!FDPH_IDX((long long)tk.item * 32 + 32 <= a.cap_partial, a.err)) return;
-    const double ks = (double)a.kinv;   // the window's storage scale
+    const float ks = a.kinv;   // the window's storage scale (a power of two)
     for (int u = threadIdx.x; u < nb * NR * 32; u += 32 * kTcWarps) {
         const int i = u & 31, r = (u >> 5) % NR, b = (u >> 5) / NR;
-        double s = 0.0;
+        const float* v = (const float*)tc_smem + (size_t)(b * NR + r) * 32 + i;
+        double s = wide(v[0] * ks);
 #pragma unroll
-        for (int w = 0; w < kTcWarps; ++w) s += (double)((float*)tc_smem)[((size_t)w * B * NR + b * NR + r) * 32 + i] * ks;
+        for (int w = 1; w < kTcWarps; ++w) s += wide(v[(size_t)w * B * NR * 32] * ks);
         if (i < nr) a.partial[r * a.rs_partial + b * a.cap_partial + (size_t)tk.item * 32 + i] = s;
     }
 }
