@@ -1138,15 +1138,17 @@ static int build_near_begin(fdph_plan_t P, const PlanInputs& in, NearBuild& nb) 
         }
         FDPH_CUDA(cudaMemcpyAsync(d_ms, ms.data(), npairs * sizeof(int), cudaMemcpyHostToDevice, P->stream));
     }
-    // work-item length: the longest chunk that still yields about four items per resident warp slot
-    // (152 SMs x 16), so small problems (the plain N = 256 march) fill the device too
+    // work-item length: the longest chunk that still yields about four items per resident warp
+    // (152 SMs x 16) or CTA (152 x 3), so small problems (the plain N = 256 march) fill the device too
     long long slices = 0;
     for (int l = 0; l < nl; ++l) {
         kz[l] = std::min(kz[l], W[l]);
         slices += std::max(W[l] - kz[l], 1);
     }
+    // (an item is a CTA's work on the tensor cores: FP64 plans, several right-hand sides with FP16 windows)
+    const bool cta = P->precision == FDPH_FP64 || (P->precision == FDPH_FP16 && P->nrhs >= 2);
     int chunk = std::min(near_max_chunk(P->nrhs, P->precision), kChunk / 2);
-    while (chunk > 8 / std::min(P->nrhs, 2) && slices * P->nrhs / chunk < 4LL * 152 * 16) chunk /= 2;
+    while (chunk > 8 / std::min(P->nrhs, 2) && slices * P->nrhs / chunk < 4LL * 152 * (cta ? 3 : 16)) chunk /= 2;
     finish_near_layout(hp, W, kz, has_tail, chunk, 16 / (int)sizeof(H), 16 / (int)sizeof(A), kAuxChunk);
     P->near_W = W;
     P->near_kz = kz;
@@ -1223,6 +1225,11 @@ static int build_near_begin(fdph_plan_t P, const PlanInputs& in, NearBuild& nb) 
     return FDPH_OK;
 }
 
+// near leaves that act within a rupture block, and what rec_tensor keeps of one: its kernel steps below
+// kBlk, and the static tile of a shorter window
+static bool rec_leaf(const NearLeaf& L) { return L.kz < kBlk || (L.W < kBlk && L.tail < 0); }
+static long long rec_size(const NearLeaf& L) { return L.W < kBlk ? (long long)L.W * L.sl + L.sla : (long long)kBlk * L.sl; }
+
 template <class T, class H>
 static int build_near_finish(fdph_plan_t P, const PlanInputs& in, NearBuild& nb) {
     using A = typename NearTypes<H>::Aux;
@@ -1269,15 +1276,18 @@ static int build_near_finish(fdph_plan_t P, const PlanInputs& in, NearBuild& nb)
     if constexpr (sizeof(H) == 8) {
         // the rupture leaves' first kernel steps stay as numbers; then all slices take the form of fixed.cuh
         for (const NearLeaf& L : hp.near)
-            if (L.kz < kBlk) P->rec_len += (long long)std::min(L.W, kBlk) * L.sl;
+            if (rec_leaf(L)) P->rec_len += rec_size(L);
         if ((rc = dalloc(P, &P->rec_tensor, (size_t)P->rec_len))) return rc;
         long long at = 0;
         for (const NearLeaf& L : hp.near)
-            if (L.kz < kBlk) {
+            if (rec_leaf(L)) {
                 const size_t c = (size_t)std::min(L.W, kBlk) * L.sl;
                 if (c) FDPH_CUDA(cudaMemcpyAsync(P->rec_tensor + at, (const double*)P->tensor + L.tensor, c * sizeof(double),
                                                  cudaMemcpyDeviceToDevice, P->stream));
-                at += (long long)c;
+                if (L.W < kBlk)
+                    FDPH_CUDA(cudaMemcpyAsync(P->rec_tensor + at + c, (const double*)P->stat + L.stat, L.sla * sizeof(double),
+                                              cudaMemcpyDeviceToDevice, P->stream));
+                at += rec_size(L);
             }
         std::vector<long long> win0, aux0;
         slice_numbers(hp, win0, aux0);
@@ -1300,15 +1310,16 @@ static int build_near_finish(fdph_plan_t P, const PlanInputs& in, NearBuild& nb)
 // Rupture blocks: the near leaves that a wave crosses within kBlk steps, grouped by their maximal
 // receiver clusters (clusters of one tree are nested or disjoint, so those are disjoint; every element
 // is in one, its own leaf has kz = 0), and whether blocks may be longer than one step: nothing else may
-// act within the block, so the far blocks need min(dm + delay) >= kBlk, and the static and tail terms,
-// which start at the window's end, W >= kBlk.
+// act within the block, so the far blocks need min(dm + delay) >= kBlk, and tail terms, which start at the
+// window's end, W >= kBlk (the static terms of shorter windows are among the block's own).
 static int build_recent(fdph_plan_t P) {
     const HostPlan& hp = P->hp;
-    bool far_late = P->margin >= kBlk, near_late = true;
+    const bool far_late = P->margin >= kBlk;
+    bool near_late = true;
     std::vector<int> use;
     for (int l = 0; l < (int)hp.near.size(); ++l) {
-        near_late = near_late && hp.near[l].W >= kBlk;
-        if (hp.near[l].kz < kBlk) use.push_back(l);
+        near_late = near_late && (hp.near[l].W >= kBlk || hp.near[l].tail < 0);
+        if (rec_leaf(hp.near[l])) use.push_back(l);
     }
     P->rup_block = far_late && near_late && P->far_mode == 0 ? kBlk : 1;
     std::vector<int> owner(hp.n, -1);      // first element of the largest receiver range over each element
@@ -1336,7 +1347,7 @@ static int build_recent(fdph_plan_t P) {
         long long o = 0;
         for (int l : use) {
             at[l] = o;
-            o += (long long)std::min(hp.near[l].W, kBlk) * hp.near[l].sl;
+            o += rec_size(hp.near[l]);
         }
     }
     for (size_t g = 0; g < groups.size(); ++g) {
@@ -1344,7 +1355,8 @@ static int build_recent(fdph_plan_t P) {
         groups[g].nleaf = (int)per[g].size();
         for (int l : per[g]) {
             const NearLeaf& L = hp.near[l];
-            leaves.push_back({P->rec_tensor ? at[l] : (long long)L.tensor, L.sl, L.r0, L.nr, L.s0, L.ns, L.kz, L.W, {0, 0, 0}});
+            const long long stat = L.W < kBlk && L.tail < 0 ? (P->rec_tensor ? at[l] + (long long)L.W * L.sl : (long long)L.stat) : -1;
+            leaves.push_back({P->rec_tensor ? at[l] : (long long)L.tensor, stat, L.sl, L.r0, L.nr, L.s0, L.ns, L.kz, L.W, 0});
         }
     }
     P->n_groups = (int)groups.size();

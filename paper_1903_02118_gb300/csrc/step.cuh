@@ -90,8 +90,9 @@ struct RecGroup {
     int r0, nr, leaf0, nleaf;
 };
 struct __align__(16) RecLeaf {
-    long long off;       // element offset of kernel step 0
-    int sl, r0, nr, s0, ns, kz, W, pad[3];
+    long long off;       // element offset of kernel step 0 in rec_tensor
+    long long stat;      // W < kBlk: the static tile, in rec_tensor (FP64) or the aux slices; else -1
+    int sl, r0, nr, s0, ns, kz, W, pad;
 };
 static_assert(sizeof(RecLeaf) == 48, "a leaf is three 16-byte loads");
 
@@ -886,9 +887,10 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
             const bool on = ai < tk.k1 && in;
             if (on && ai == 0) {
 #pragma unroll
-                for (int b = 0; b < B; ++b)
-                    vr[b * (span + 4) + ri] =
-                        narrow(b < nb && src && t0 + b >= 0 ? Cr[(size_t)wrap(t0 + b, a.WC) * a.N] : 0.0, R());
+                for (int b = 0; b < B; ++b) {
+                    const int t = min(t0 + b, hend - 1);   // (the slip by the steps that the launch may use)
+                    vr[b * (span + 4) + ri] = narrow(b < nb && src && t >= 0 ? Cr[(size_t)wrap(t, a.WC) * a.N] : 0.0, R());
+                }
             } else if (on) {
                 const double rho = a.rho[ai - 1];
                 double v = src ? vs[(size_t)(ai - 1) * ns] : 0.0;
@@ -953,7 +955,8 @@ struct FrictionDev {
 // slip rates before the step's aligned block [n0, n0 + kBlk) do, computed for the whole block
 // beforehand) plus what the block's own earlier steps n0 ... n - 1 do: by causality only the kernel
 // steps 1 ... n - n0 of the near leaves that a wave crosses that fast (RecLeaf: the first kz kernel
-// steps of a leaf vanish; the far blocks and the static and tail terms act later than kBlk steps, see
+// steps of a leaf vanish), and the static term of leaves with a window shorter than a block, on the slip
+// C(n - W) - C(n0 - 1) (the far blocks and the other static and tail terms act later than kBlk steps, see
 // rup_block).  One CTA per receiver group (the disjoint maximal receiver clusters of those leaves): its
 // warps take the (leaf, kernel step) units in turn, then the first warp solves the friction law and
 // appends the slip rate (push).  b: the step within the launch sequence's block.
@@ -993,25 +996,29 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
         k0 = f.k0[e];
     }
     __syncthreads();
-    auto leaf = [&](int q) -> RecLeaf { return q < kRupLeaves ? leaves[q] : a.rec_leaves[g.leaf0 + q]; };
-    auto range = [&](const RecLeaf& L, int& first) {
+    auto leaf = [&](int q) -> const RecLeaf& { return q < kRupLeaves ? leaves[q] : a.rec_leaves[g.leaf0 + q]; };
+    // units of a leaf: its kernel steps first, first + 1, ..., then (kernel step -1) its static term
+    auto range = [&](const RecLeaf& L, int& first, int& steps) {
         first = max(L.kz, 1);
-        return max(min(back + 1, L.W) - first, 0);   // kernel steps first, first + 1, ...
+        steps = max(min(back + 1, L.W) - first, 0);
+        return steps + (L.stat >= 0 && back >= max(L.W, 1) ? 1 : 0);
     };
     // the unit with running number r from leaf q on: its leaf (nleaf: none) and kernel step
-    auto seek = [&](int& q, int r, RecLeaf& L, int& k) {
+    auto seek = [&](int& q, int r, int& k) {
         for (; q < g.nleaf; ++q) {
-            int first;
-            L = leaf(q);
-            const int len = range(L, first);
+            int first, steps;
+            const int len = range(leaf(q), first, steps);
             if (r < len) {
-                k = first + r;
+                k = r < steps ? first + r : -1;
                 return;
             }
             r -= len;
         }
     };
+    using A = typename NearTypes<H>::Aux;
+    constexpr int VA = 16 / (int)sizeof(A);
     auto load_x = [&](const RecLeaf& L, int k, uint4 (&x)[NB]) {
+        if (k < 0) return;   // (a static tile is read where it is used)
         const H* sl = (const H*)a.rec_tensor + L.off + (size_t)k * L.sl + (size_t)(lane < L.nr ? lane : 0) * V;
         const bool in = FDPH_IDX(L.off + (long long)(k + 1) * L.sl <= a.len_rec, a.err);
 #pragma unroll
@@ -1019,16 +1026,22 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
             x[jb] = in && jb * V < L.ns ? *(const uint4*)(sl + (size_t)jb * L.nr * V) : make_uint4(0, 0, 0, 0);
     };
     auto load_v = [&](const RecLeaf& L, int k) -> R {
-        const size_t off = (size_t)wrap(n - k, a.WD) * a.N + L.s0 + min(lane, L.ns - 1);
+        const int c = L.s0 + min(lane, L.ns - 1);
         R v;
-        if constexpr (sizeof(R) == 4) v = a.Dring32[off]; else v = a.Dring[off];
+        if (k < 0) {   // the slip of the block's steps up to n - W
+            const int t = min(n - L.W, n - 1), t0 = n - back - 1;
+            const double before = t0 >= 0 ? a.Cring[(size_t)wrap(t0, a.WC) * a.N + c] : 0.0;
+            v = narrow(a.Cring[(size_t)wrap(t, a.WC) * a.N + c] - before, R());
+        } else {
+            const size_t off = (size_t)wrap(n - k, a.WD) * a.N + c;
+            if constexpr (sizeof(R) == 4) v = a.Dring32[off]; else v = a.Dring[off];
+        }
         return lane < L.ns ? v : (R)0;
     };
-    RecLeaf L;
     int q = 0, k = 0;
     uint4 x[NB];
-    seek(q, warp, L, k);
-    if (q < g.nleaf) load_x(L, k, x);
+    seek(q, warp, k);
+    if (q < g.nleaf) load_x(leaf(q), k, x);
     cudaGridDependencySynchronize();                 // the step before is complete
     cudaTriggerProgrammaticLaunchCompletion();
     double u = 0.0, c = 0.0, comp = 0.0;
@@ -1037,33 +1050,49 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
         c = a.C[p];
         comp = a.Ccomp[p];
     }
-    R v = q < g.nleaf ? load_v(L, k) : (R)0;
+    R v = q < g.nleaf ? load_v(leaf(q), k) : (R)0;
     for (int buf = 0; q < g.nleaf; buf ^= 1) {
         row[warp][buf][lane] = v;
         __syncwarp();
+        const RecLeaf& L = leaf(q);
         const int ns = L.ns, nr = L.nr, r0 = L.r0 - g.r0;
+        R s = 0;
+        const bool fixed = k < 0;
+        if (fixed) {
+            const A* sl = (const A*)(sizeof(H) == 8 ? a.rec_tensor : a.stat) + L.stat + (size_t)(lane < nr ? lane : 0) * VA;
+            const bool in = FDPH_IDX(L.stat + (long long)((ns + VA - 1) / VA) * VA * nr <= (sizeof(H) == 8 ? a.len_rec : a.len_aux), a.err);
+            for (int jb = 0; jb * VA < ns && in; ++jb) {
+                R xv[VA], y[VA];
+                unpack(*(const uint4*)(sl + (size_t)jb * nr * VA), xv, R());
+                load_row<VA>(&row[warp][buf][jb * VA], y);
+#pragma unroll
+                for (int i = 0; i < VA; ++i) s = fma(xv[i], y[i], s);
+            }
+        }
         // the unit W further: its slip rates are loaded meanwhile, its coefficients next
         {
-            int first;
-            range(L, first);
-            seek(q, k - first + W, L, k);
+            int first, steps;
+            range(L, first, steps);
+            seek(q, (fixed ? steps : k - first) + W, k);
         }
-        if (q < g.nleaf) v = load_v(L, k);
-        R s = 0;
+        if (q < g.nleaf) v = load_v(leaf(q), k);
+        if (!fixed) {
 #pragma unroll
-        for (int jb = 0; jb < NB; ++jb) {
-            if (jb * V >= ns) break;
-            R xv[V], y[V];
-            if constexpr (sizeof(H) == 2) unpack(x[jb], xv, __half());
-            else unpack(x[jb], xv, R());
-            load_row<V>(&row[warp][buf][jb * V], y);
-            R t = xv[0] * y[0];
+            for (int jb = 0; jb < NB; ++jb) {
+                if (jb * V >= ns) break;
+                R xv[V], y[V];
+                if constexpr (sizeof(H) == 2) unpack(x[jb], xv, __half());
+                else unpack(x[jb], xv, R());
+                load_row<V>(&row[warp][buf][jb * V], y);
+                R t = xv[0] * y[0];
 #pragma unroll
-            for (int i = 1; i < V; ++i) t = fma(xv[i], y[i], t);
-            s += t;
+                for (int i = 1; i < V; ++i) t = fma(xv[i], y[i], t);
+                s += t;
+            }
+            s *= (R)a.kinv;   // (the window's storage scale, a power of two)
         }
-        if (q < g.nleaf) load_x(L, k, x);
-        if (lane < nr && FDPH_IDX(r0 >= 0 && r0 + nr <= 32, a.err)) red[warp][r0 + lane] += wide(s * (R)a.kinv);
+        if (q < g.nleaf) load_x(leaf(q), k, x);
+        if (lane < nr && FDPH_IDX(r0 >= 0 && r0 + nr <= 32, a.err)) red[warp][r0 + lane] += wide(s);
         __syncwarp();
     }
     __syncthreads();

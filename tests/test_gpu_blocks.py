@@ -128,3 +128,40 @@ def test_cut_ruptures_give_the_same_bits(prec, leaf, eps_st, cfl):
     assert (outs[0][0] > 0).mean() > 0.05
     for o in outs[1:]:
         assert all(np.array_equal(x, y) for x, y in zip(o, outs[0]))
+
+
+@pytest.mark.parametrize("prec,eps_st,cfl", [(fdph.FP64, 0.05, 0.5), (fdph.FP32, 1e-3, 0.25), (fdph.FP64, 1e-3, 0.25)])
+def test_short_windows_rupture_equals_predict_and_commit(prec, eps_st, cfl):
+    """Leaves whose window is shorter than a block: their static terms act within the block.  Against the
+    same law solved by the caller between predict and commit (FP64 to rounding, FP32 products to 1e-5)."""
+    _need_gpu()
+    N, M = 240, 100
+    plan = fdph.Plan(inputs.kinked_fault(N), cfl, M, 1e-6, eta=0.5, eps_st=eps_st, leaf_size=16, precision=prec)
+    tau0 = np.full(N, 0.45)
+    tau0[N // 2 - 8:N // 2 + 8] = 0.61
+    t0 = torch.from_numpy(tau0).cuda()
+    plan.rupture_init(t0, 1.0, 0.6, 0.3, 2.0)
+    D = torch.zeros((M, N), dtype=torch.float64, device="cuda")
+    T = torch.zeros_like(D)
+    torch.cuda.synchronize()
+    plan.rupture_run(M, D, T)
+    plan.synchronize()
+    plan.reset()
+    k0 = torch.from_numpy(plan.self_coefficients()).cuda()
+    slip = torch.zeros(N, dtype=torch.float64, device="cuda")
+    Du, Tu = torch.zeros_like(D), torch.zeros_like(T)
+    for n in range(M):
+        plan.predict(Tu[n])
+        plan.synchronize()
+        tau = t0 + Tu[n]
+        strength = 0.6 - 0.3 * torch.clamp(slip / 2.0, max=1.0)
+        v = torch.where(tau > strength, (tau - strength) / (-k0), torch.zeros_like(tau))
+        Du[n] = v
+        Tu[n] = tau + k0 * v
+        slip += v * cfl
+        torch.cuda.synchronize()
+        plan.commit(Du[n])
+    plan.synchronize()
+    tol = 1e-10 if prec == fdph.FP64 else 1e-5
+    assert (D > 0).double().mean().item() > 0.05
+    assert ((D - Du).norm() / Du.norm()).item() < tol and ((T - Tu).norm() / Tu.norm()).item() < tol
