@@ -115,8 +115,13 @@ static inline int near_max_chunk(int nrhs, int precision) {
     return (nrhs >= 2 && precision != FDPH_FP64 ? 2 * kChunk : kChunk) / nrhs;
 }
 
-// the longest aux item (static tile and tail slices): all of a leaf's
-static const int kAuxChunk = 1 + kMaxSoe;
+// the longest aux item: all of a leaf's static tile and tail slices, or half of them where one warp takes an
+// item and there is less than one leaf per scheduler (152 SMs x 4): one item of all 17 slices then takes as
+// long as the rest of the step (curved N = 1024, 422 leaves: 0.95 -> 0.80 ms per 64 steps; with 1963 leaves the
+// split costs 2.18 -> 2.38 ms)
+static inline int near_aux_chunk(int precision, int leaves) {
+    return precision == FDPH_FP64 || leaves >= 4 * 152 ? 1 + kMaxSoe : 9;
+}
 
 // ------------------------------------------------------------------------------------------
 // plan-time device kernels: near-field windows and exact-kernel tensors
@@ -278,6 +283,7 @@ struct fdph_plan_s {
     void* fac = nullptr;
     int *ints = nullptr, *src_order = nullptr;
     int4 *runs = nullptr, *sc_tasks = nullptr;
+    int* last_run = nullptr;
     int n_sct = 0;
     FarEnt* ents = nullptr;
     double* ent_phi = nullptr;
@@ -312,7 +318,6 @@ struct fdph_plan_s {
     // state
     double *Dring = nullptr, *Cring = nullptr, *C = nullptr, *Ccomp = nullptr;
     float* Dring32 = nullptr;   // FP32 copy of Dring (FP32 / FP16 plans)
-    float* Dscale = nullptr;    // its rows' inverse scales (tensor-core near field)
     double *tfar = nullptr, *thist = nullptr, *blkD = nullptr, *blkC = nullptr;   // a block's scratch
     std::vector<std::pair<unsigned char*, size_t>> canaries;   // FDPH_CHECK builds: allocation ends
     double *ring = nullptr, *zring = nullptr, *partial = nullptr;
@@ -344,6 +349,7 @@ struct fdph_plan_s {
     std::vector<int32_t> near_W, near_kz;
     std::vector<char> near_tail;
     int chunk = 0;            // steps of exact kernel per near-field work item
+    int aux_chunk = 1;        // aux slices per work item
     double kscale = 1.0;      // FP16 window coefficients are stored as K * kscale (a power of two)
     int sched_version = 0;    // bumped whenever the near-field items are rebuilt
     size_t partial_cap = 0;   // capacity of `partial`, in doubles
@@ -434,7 +440,6 @@ static StepArgs<T> make_args(fdph_plan_t P, const double* D, double* T_) {
     a.perm = P->perm;
     a.Dring = P->Dring;
     a.Dring32 = P->Dring32;
-    a.Dscale = P->Dscale;
     a.Cring = P->Cring;
     a.C = P->C;
     a.Ccomp = P->Ccomp;
@@ -446,6 +451,7 @@ static StepArgs<T> make_args(fdph_plan_t P, const double* D, double* T_) {
     a.runs = P->runs;
     a.src_order = P->src_order;
     a.sc_tasks = P->sc_tasks;
+    a.last_run = P->last_run;
     a.n_sct = P->n_sct;
     a.ents = P->ents;
     a.ent_phi = P->ent_phi;
@@ -566,54 +572,47 @@ static void launch_near_items(const StepArgs<T>& a, int chunk, cudaStream_t s) {
         a, (int)wb);
 }
 
-// the tensor-core window items of a launch's steps, B steps at a time
+// the tensor-core window items
 template <int NR, int B>
-static void launch_tc(StepArgs<float> a, int n_win, int chunk, cudaStream_t s) {
-    const int nb = a.nb, n_off = a.n_off;
-    double* partial = a.partial;
-    for (int b = 0; b < nb; b += B) {
-        a.n_off = n_off + b;
-        a.nb = std::min(B, nb - b);
-        a.partial = partial + b * a.cap_partial;
-        tc_block_kernel<NR, B><<<n_win, 32 * kTcWarps, TcCfg<NR, B>::smem(chunk), s>>>(a);
-    }
+static void launch_tc(const StepArgs<float>& a, int n_win, int chunk, cudaStream_t s) {
+    tc_block_kernel<NR, B><<<n_win, 32 * TcCfg<NR, B>::warps, TcCfg<NR, B>::smem(chunk), s>>>(a, chunk);
 }
 
-template <class T, class H>
-static void launch_near_h(fdph_plan_t P, StepArgs<T> a, cudaStream_t s) {
-    if constexpr (sizeof(H) == 8) {   // FP64: exact products on the tensor cores
-        if (!a.n_items) return;
+// The near field of a launch: the window items (FP16 plans), or all items (FP64 and FP32 plans)
+template <class T>
+static void launch_near(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
+    if (!a.n_items) return;
+    if constexpr (sizeof(T) == 8) {   // exact products on the tensor cores
         const dim3 g(a.n_items, a.nrhs);
         if (a.nb == 1) fixed_block_kernel<1><<<g, 32 * kFxWarps, FxCfg<1>::smem(P->chunk), s>>>(a, P->chunk);
         else fixed_block_kernel<kBlk><<<g, 32 * kFxWarps, FxCfg<kBlk>::smem(P->chunk), s>>>(a, P->chunk);
-        return;
-    } else {
-    if constexpr (std::is_same<H, __half>::value) {
-        if (P->nrhs >= 2) {
-            if (P->n_win) {
-                if (P->nrhs == 2) a.nb == 1 ? launch_tc<2, 2>(a, P->n_win, P->chunk, s) : launch_tc<2, 16>(a, P->n_win, P->chunk, s);
-                else if (P->nrhs == 4) a.nb == 1 ? launch_tc<4, 1>(a, P->n_win, P->chunk, s) : launch_tc<4, 8>(a, P->n_win, P->chunk, s);
-                else a.nb == 1 ? launch_tc<8, 1>(a, P->n_win, P->chunk, s) : launch_tc<8, 8>(a, P->n_win, P->chunk, s);
-            }
-            a.tasks += P->n_win;
-            a.n_items = P->n_aux;
+    } else if (P->precision == FDPH_FP16) {
+        if (!P->n_win) return;
+        const bool one = a.nb == 1;
+        switch (P->nrhs) {
+            case 2: one ? launch_tc<2, 1>(a, P->n_win, P->chunk, s) : launch_tc<2, kBlk>(a, P->n_win, P->chunk, s); break;
+            case 4: one ? launch_tc<4, 1>(a, P->n_win, P->chunk, s) : launch_tc<4, kBlk>(a, P->n_win, P->chunk, s); break;
+            case 8: one ? launch_tc<8, 1>(a, P->n_win, P->chunk, s) : launch_tc<8, kBlk>(a, P->n_win, P->chunk, s); break;
+            default: one ? launch_tc<1, 1>(a, P->n_win, P->chunk, s) : launch_tc<1, kBlk>(a, P->n_win, P->chunk, s);
         }
-    }
-    if (!a.n_items) return;
-    if (a.nb == 1) launch_near_items<T, H, 1>(a, P->chunk, s);
-    else launch_near_items<T, H, kBlk>(a, P->chunk, s);
+    } else if (a.nb == 1) {
+        launch_near_items<T, float, 1>(a, P->chunk, s);
+    } else {
+        launch_near_items<T, float, kBlk>(a, P->chunk, s);
     }
 }
 
+// The static and tail items of FP16 plans: a kernel of their own, far from filling the GPU, so it goes last
+// on the far-field branch, beside the windows
 template <class T>
-static void launch_near(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
+static void launch_near_aux(fdph_plan_t P, StepArgs<T> a, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
-        if (P->precision == FDPH_FP16) {
-            launch_near_h<T, __half>(P, a, s);
-            return;
-        }
+        if (P->precision != FDPH_FP16 || !P->n_aux) return;
+        a.tasks += P->n_win;
+        a.n_items = P->n_aux;
+        if (a.nb == 1) launch_near_items<T, __half, 1>(a, P->chunk, s);
+        else launch_near_items<T, __half, kBlk>(a, P->chunk, s);
     }
-    launch_near_h<T, T>(P, a, s);
 }
 
 // The part of a block that only reads slip rates and rings: transient convolution and Eq. 39 beside the
@@ -631,11 +630,7 @@ static void enqueue_far(const StepArgs<T>& a, cudaStream_t s) {
 // causality), and then a second branch; otherwise they follow.
 template <class T>
 static void enqueue_block(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
-    {
-        ProfScope ps(P, 0, a.nb);
-        push_kernel<T><<<dim3(blocks(a.N, 128), a.nrhs), 128, 0, s>>>(a);
-        if (a.Dscale) row_scale_kernel<T><<<dim3(a.nb, a.nrhs), kRowThreads, 0, s>>>(a, 0);
-    }
+    { ProfScope ps(P, 0, a.nb); push_kernel<T><<<dim3(blocks(a.N, 128), a.nrhs), 128, 0, s>>>(a); }
     if (!P->prof) {
         const bool apart = a.nb <= P->margin;
         cudaStream_t f0 = P->side[0], f1 = apart ? P->side[1] : P->side[0];
@@ -646,6 +641,7 @@ static void enqueue_block(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
         if (a.n_fir) launch_fir<T>(a, f0);
         launch_eq42<T>(a, f0);
         enqueue_far<T>(a, f1);
+        launch_near_aux<T>(P, a, f1);
         cudaEventRecord(P->ev_join[0], f0);
         cudaStreamWaitEvent(s, P->ev_join[0], 0);
         if (apart) {
@@ -659,7 +655,7 @@ static void enqueue_block(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
     if (a.n_fir) { ProfScope ps(P, 1, a.nb); launch_fir<T>(a, s); }
     { ProfScope ps(P, 2, a.nb); launch_eq42<T>(a, s); }
     if (a.n_tr) { ProfScope ps(P, 3, a.nb); launch_trconv<T>(a, s); }
-    { ProfScope ps(P, 4, a.nb); launch_near<T>(P, a, s); }
+    { ProfScope ps(P, 4, a.nb); launch_near<T>(P, a, s); launch_near_aux<T>(P, a, s); }
     { ProfScope ps(P, 5, a.nb); launch_far<T>(a, s); launch_gather<T>(a, s); }
 }
 
@@ -673,13 +669,14 @@ static void enqueue_history(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s)
         cudaStreamWaitEvent(P->side[1], P->ev_fork, 0);
         launch_near<T>(P, a, s);
         enqueue_far<T>(a, P->side[1]);
+        launch_near_aux<T>(P, a, P->side[1]);
         cudaEventRecord(P->ev_join[1], P->side[1]);
         cudaStreamWaitEvent(s, P->ev_join[1], 0);
         launch_gather<T>(a, s);
         return;
     }
     if (a.n_tr) { ProfScope ps(P, 3, a.nb); launch_trconv<T>(a, s); }
-    { ProfScope ps(P, 4, a.nb); launch_near<T>(P, a, s); }
+    { ProfScope ps(P, 4, a.nb); launch_near<T>(P, a, s); launch_near_aux<T>(P, a, s); }
     { ProfScope ps(P, 5, a.nb); launch_far<T>(a, s); launch_gather<T>(a, s); }
 }
 
@@ -972,7 +969,7 @@ template <class T, class H>
 static int build_schedule(fdph_plan_t P) {
     using A = typename NearTypes<H>::Aux;
     HostPlan& hp = P->hp;
-    const bool tc = std::is_same<H, __half>::value && P->nrhs >= 2;
+    const bool tc = std::is_same<H, __half>::value;
     const int ni = (int)hp.items.size();
     std::vector<NearTask> all(ni);
     std::vector<double> cost(ni);
@@ -1010,12 +1007,14 @@ static int build_schedule(fdph_plan_t P) {
     for (int q = 0; q < ni; ++q) tasks[q] = all[order[q]];
     // shared memory of the near kernels for items of this length
     if (tc) {
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<2, 2>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<2, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<2, 16>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<1, 1>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<1, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<1, kBlk>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<2, 1>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<2, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<2, kBlk>::smem(kChunk)));
         FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<4, 1>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<4, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<4, 8>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<4, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<4, kBlk>::smem(kChunk)));
         FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8, 1>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8, 8>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8, kBlk>::smem(kChunk)));
     }
     if constexpr (sizeof(H) == 8) {
         FDPH_CUDA(cudaFuncSetAttribute(fixed_block_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FxCfg<1>::smem(kChunk)));
@@ -1145,11 +1144,12 @@ static int build_near_begin(fdph_plan_t P, const PlanInputs& in, NearBuild& nb) 
         kz[l] = std::min(kz[l], W[l]);
         slices += std::max(W[l] - kz[l], 1);
     }
-    // (an item is a CTA's work on the tensor cores: FP64 plans, several right-hand sides with FP16 windows)
-    const bool cta = P->precision == FDPH_FP64 || (P->precision == FDPH_FP16 && P->nrhs >= 2);
+    // (an item is a CTA's work on the tensor cores: FP64 and FP16 plans)
+    const bool cta = P->precision != FDPH_FP32;
     int chunk = std::min(near_max_chunk(P->nrhs, P->precision), kChunk / 2);
     while (chunk > 8 / std::min(P->nrhs, 2) && slices * P->nrhs / chunk < 4LL * 152 * (cta ? 3 : 16)) chunk /= 2;
-    finish_near_layout(hp, W, kz, has_tail, chunk, 16 / (int)sizeof(H), 16 / (int)sizeof(A), kAuxChunk);
+    P->aux_chunk = near_aux_chunk(P->precision, nl);
+    finish_near_layout(hp, W, kz, has_tail, chunk, 16 / (int)sizeof(H), 16 / (int)sizeof(A), P->aux_chunk);
     P->near_W = W;
     P->near_kz = kz;
     P->near_tail = has_tail;
@@ -1451,7 +1451,7 @@ static int set_chunk(fdph_plan_t P, int chunk) {
     FDPH_CUDA(cudaStreamSynchronize(P->stream));
     drop_graphs(P);
     const int64_t tens0 = hp.near_tensor_len, aux0 = hp.near_aux_len, vst0 = hp.vstate_len;
-    finish_near_layout(hp, P->near_W, P->near_kz, P->near_tail, chunk, 16 / (int)sizeof(H), 16 / (int)sizeof(A), kAuxChunk);
+    finish_near_layout(hp, P->near_W, P->near_kz, P->near_tail, chunk, 16 / (int)sizeof(H), 16 / (int)sizeof(A), P->aux_chunk);
     if (hp.near_tensor_len != tens0 || hp.near_aux_len != aux0 || hp.vstate_len != vst0) {
         // the stored coefficients and states must keep their places (only the items change)
         set_error("set_chunk: near-field layout changed; the plan is unusable");
@@ -1842,6 +1842,7 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
     std::vector<int4> sct, runs(hp.run_delay.size());
     for (size_t q = 0; q < runs.size(); ++q)
         runs[q] = make_int4(hp.run_delay[q], hp.run_len[q], hp.run_start[q], hp.src_order[hp.run_start[q]]);
+    std::vector<int> last_run;   // per ring slot: the last run with delay <= the slot's offset
     P->margin = INT32_MAX;
     for (size_t q = 0; q < hp.sbs.size(); ++q) {
         const SubBlock& b = hp.sbs[q];
@@ -1850,11 +1851,12 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
         int lg = 0;
         while ((1 << lg) < std::min(b.rank, 32)) ++lg;
         if (b.ident == 2) lg = 0;
-        const int S = 32 >> lg;
-        int last = b.run0;   // the last run with delay <= the warp's last slot
-        for (int d = b.mindelay; d <= b.maxdelay + kBlk - 1; d += S) {
-            while (last + 1 < b.run0 + b.nruns && hp.run_delay[last + 1] <= d + S - 1) ++last;
-            sct.push_back(make_int4((int)q, d, last, lg));
+        const int S = 32 >> lg, d1 = b.maxdelay + kBlk - 1;
+        for (int d = b.mindelay; d <= d1; d += S) sct.push_back(make_int4((int)q, d, (int)last_run.size() + d - b.mindelay, lg));
+        int last = b.run0;
+        for (int d = b.mindelay; d <= d1; ++d) {
+            while (last + 1 < b.run0 + b.nruns && hp.run_delay[last + 1] <= d) ++last;
+            last_run.push_back(last);
         }
     }
     P->n_sct = (int)sct.size();
@@ -1868,6 +1870,21 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
         ents[e] = {tr ? (long long)b.zring : (long long)b.ring, b.ident == 1 ? il : (long long)b.f + (long long)il * b.rank,
                    tr ? b.LZ : b.L, hp.ints[b.dm + il], b.rank, (tr ? 1 : 0) | (b.ident == 1 ? 2 : 0)};
         if (hp.interp) ephi[e] = hp.phis[b.phi + il];
+    }
+    // (the lanes of a warp take entries of equal rank as far as possible)
+    for (int p = 0; p < hp.n; ++p) {
+        const int e0 = hp.g_ptr[p], e1 = hp.g_ptr[p + 1];
+        std::vector<int> ord(e1 - e0);
+        for (int e = e0; e < e1; ++e) ord[e - e0] = e;
+        std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return ents[x].rank < ents[y].rank; });
+        std::vector<FarEnt> es(e1 - e0);
+        std::vector<double> ps(e1 - e0);
+        for (int k = 0; k < e1 - e0; ++k) {
+            es[k] = ents[ord[k]];
+            if (hp.interp) ps[k] = ephi[ord[k]];
+        }
+        std::copy(es.begin(), es.end(), ents.begin() + e0);
+        if (hp.interp) std::copy(ps.begin(), ps.end(), ephi.begin() + e0);
     }
     P->n_ent = (long long)ents.size();
     // FIR: the tasks of a source element in groups of 32, waveforms interleaved over a group's lanes
@@ -1903,7 +1920,7 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
             for (int m = 0; m < b.taps; ++m) fh[(size_t)g.h + (size_t)m * 32 + c] = hp.fac[b.h + (size_t)hp.fir_j[t] * b.taps + m];
         }
     }
-    if ((rc = upload(P, &P->sc_tasks, sct)) || (rc = upload(P, &P->runs, runs)) || (rc = upload(P, &P->ents, ents)) ||
+    if ((rc = upload(P, &P->sc_tasks, sct)) || (rc = upload(P, &P->runs, runs)) || (rc = upload(P, &P->last_run, last_run)) || (rc = upload(P, &P->ents, ents)) ||
         (rc = upload(P, &P->fir, fir)) || (rc = upload(P, &P->fir_dhat, fdh)))
         return fail(rc);
     if (hp.interp && (rc = upload(P, &P->ent_phi, ephi))) return fail(rc);
@@ -1977,11 +1994,6 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
         if ((rc = dalloc(P, &P->Dring32, c))) return fail(rc);
         sb += c * 4;
     }
-    if (P->precision == FDPH_FP16 && P->nrhs >= 2) {   // row scales of the tensor-core near field
-        const size_t c = (size_t)P->WD * P->nrhs;
-        if ((rc = dalloc(P, &P->Dscale, c))) return fail(rc);
-        sb += c * 4;
-    }
     P->state_bytes = sb;
     P->partial_cap = std::max<size_t>(hp.items.size() * 32, 1);
     if ((rc = fdph_reset(P))) return fail(rc);
@@ -2003,7 +2015,6 @@ int fdph_reset(fdph_plan_t P) {
             FDPH_CUDA(cudaMemsetAsync(bufs[q], 0, std::max<size_t>(cnt[q], 1) * P->nrhs * sizeof(double), P->stream));
     if (P->Dring32)
         FDPH_CUDA(cudaMemsetAsync(P->Dring32, 0, (size_t)P->WD * P->N * P->nrhs * sizeof(float), P->stream));
-    if (P->Dscale) FDPH_CUDA(cudaMemsetAsync(P->Dscale, 0, (size_t)P->WD * P->nrhs * sizeof(float), P->stream));
     if (P->rupture) FDPH_CUDA(cudaMemsetAsync(P->fr.slip, 0, P->N * sizeof(double), P->stream));
     FDPH_CUDA(cudaStreamSynchronize(P->stream));
     P->n = 0;
@@ -2315,11 +2326,6 @@ int fdph_load_state(fdph_plan_t P, const void* buf, size_t len) {
     if (P->Dring32) {
         const long long c = (long long)P->WD * P->N * P->nrhs;
         ring_to_float_kernel<<<blocks(c, 256), 256, 0, P->stream>>>(P->Dring, P->Dring32, c);
-        FDPH_CUDA(cudaGetLastError());
-    }
-    if (P->Dscale) {   // every row's scale from the restored ring
-        const StepArgs<float> a = make_args<float>(P, nullptr, nullptr);
-        row_scale_kernel<float><<<dim3(P->WD, P->nrhs), kRowThreads, 0, P->stream>>>(a, 1);
         FDPH_CUDA(cudaGetLastError());
     }
     FDPH_CUDA(cudaStreamSynchronize(P->stream));   // the caller may reuse the buffer on return

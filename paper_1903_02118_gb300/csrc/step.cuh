@@ -119,7 +119,6 @@ struct StepArgs {
     const int* perm;          // internal -> geometry
     double* Dring;            // [WD][N]
     float* Dring32;           // [WD][N] FP32 copy of Dring (plans whose near-field rows are FP32)
-    float* Dscale;            // [WD][nrhs] inverse power-of-two scales of the rows (tensor-core near field)
     double* Cring;            // [WC][N]
     double* C;                // [N] cumulative slip (rounded sum)
     double* Ccomp;            // [N] Kahan compensation
@@ -130,7 +129,8 @@ struct StepArgs {
     const int* ints;
     const int4* runs;         // {delay, sources, first in src_order, first source}
     const int* src_order;
-    const int4* sc_tasks;     // scatter warp tasks {block, first slot offset, last run, log2 lanes per slot}
+    const int4* sc_tasks;     // scatter warp tasks {block, first slot offset, its place in last_run, log2 lanes per slot}
+    const int* last_run;      // per slot offset of a block: the last run with delay <= it
     int n_sct;
     const FarEnt* ents;       // Eq. 39 entries, receiver-major
     const double* ent_phi;    // sub-step receiver delays (interpolated reading; null: rounded)
@@ -441,16 +441,16 @@ __global__ void scatter_kernel(StepArgs<T> a0) {
     const int d = tk.y + (lane >> tk.w);
     const int maxdelay = sb.maxdelay, rank = sb.rank, run0 = sb.run0;
     if (d > maxdelay + nb - 1) return;
-    int run = tk.z;
-    while (run >= run0 && a.runs[run].x > d) --run;
-    if (run < run0 || d - a.runs[run].x >= nb) return;   // no step of the block comes to this slot
+    const int run = a.last_run[tk.z + (lane >> tk.w)];
+    const int4 top = a.runs[run];
+    if (d - top.x >= nb) return;   // no step of the block comes to this slot
     const int slot = wrap(n + d, sb.L);
     double* r = a.ring + sb.ring + (long long)slot * rank;
     if (!FDPH_IDX(sb.ring + (long long)(slot + 1) * rank <= a.len_ring, a.err)) return;
     if (sb.ident == 2) {
         // G is the identity: column j of a slot receives source j only, once
-        for (; run >= run0; --run) {
-            const int4 rn = a.runs[run];
+        for (int q = run; q >= run0; --q) {
+            const int4 rn = a.runs[q];
             const int b = d - rn.x;
             if (b >= nb) break;
             for (int u = lj; u < rn.y; u += G) {

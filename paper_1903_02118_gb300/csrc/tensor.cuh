@@ -1,4 +1,4 @@
-// tensor.cuh -- the near-field windows of several right-hand sides on the tensor cores (FP16 window).
+// tensor.cuh -- the near-field windows of FP16 plans on the tensor cores.
 //
 // One window slice is a 32 x 32 (receivers x sources) FP16 tile; with the R right-hand sides and the B
 // steps of a launch it meets R B slip-rate rows: a dense (32 x 32) x (32 x R B) contraction, run as
@@ -11,42 +11,23 @@
 // lane t, the A fragments of lane (g, t) are exactly the stored 16 bytes (sources 8 t ... 8 t + 7 of one
 // receiver, plan.h), and the B fragments of both 16-source steps are 16 contiguous bytes of a row.
 //
-// The slip rates must not lose digits to FP16: a row (step, right-hand side) is split into two FP16 rows
-// of x 2^sh (sh puts the row's largest entry in [2^13, 2^14); hi = fp16(x 2^sh), lo = fp16(x 2^sh - hi),
-// 2^-22 relative, 2^-39 of the row's largest entry absolute), separate columns of the contraction, so
-// that the only rounding of the FP16 path remains that of the stored coefficients.  Each slice's products
-// are scaled back per column by 2^-sh and added to the item's FP32 sums.
+// The slip rates must not lose digits to FP16: the 32 sources of a row (step, right-hand side) are split into
+// two FP16 rows of x 2^sh (sh puts the largest of them in [2^13, 2^14); hi = fp16(x 2^sh), lo =
+// fp16(x 2^sh - hi), 2^-22 relative, 2^-39 of the largest absolute), separate columns of the contraction, so
+// that the only rounding of the FP16 path remains that of the stored coefficients.  One right-hand side has
+// columns to spare and carries a third part, fp16 of what hi and lo leave: the FP32 slip rate.  Each slice's
+// products are scaled back per column by 2^-sh and added to the item's FP32 sums.  (The scale is of the
+// leaf's own sources, found by the warp that stages them: one scale for a whole step's slip rates took a
+// kernel between the push and the near field and lost digits where a leaf is quiet.)
 #pragma once
 #include "step.cuh"
 
-// Dscale[slot][right-hand side] = 2^-sh of the ring's rows: sh = 14 - e for the row's largest
-// |x| = f 2^e, f in [0.5, 1) (e from the exponent field; a zero or subnormal row takes the largest
-// shift).  One CTA per row: the launch's nb steps, or every slot (all_slots, after a state restore).
-constexpr int kRowThreads = 256;
-
-__device__ __forceinline__ int row_shift(float m) {
-    const int e = m > 0.f ? (int)((__float_as_uint(m) >> 23) & 0xffu) - 126 : -126;
-    return min(max(14 - e, -100), 100);
-}
+// the shift sh = 14 - e that takes a row's largest |x| = f 2^e, f in [0.5, 1), to [2^13, 2^14) (e from the
+// exponent field; 2^sh and 2^-sh stay normal numbers)
+__device__ __forceinline__ int row_shift(unsigned m) { return min(max(14 - ((int)(m >> 23) - 126), -115), 126); }
 
 // 2^k as a float, k in [-126, 127]
 __device__ __forceinline__ float pow2f(int k) { return __uint_as_float((unsigned)(127 + k) << 23); }
-
-template <class T>
-__global__ void __launch_bounds__(kRowThreads) row_scale_kernel(StepArgs<T> a, int all_slots) {
-    __shared__ float wmax[kRowThreads / 32];
-    const int slot = all_slots ? blockIdx.x : wrap(step_index(a) + blockIdx.x, a.WD);
-    const float* row = a.Dring32 + blockIdx.y * a.rs_D + (size_t)slot * a.N;
-    float m = 0.f;
-    for (int p = threadIdx.x; p < a.N; p += kRowThreads) m = fmaxf(m, fabsf(row[p]));
-    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < kRowThreads / 32; ++w) m = fmaxf(m, wmax[w]);
-        a.Dscale[(size_t)slot * a.nrhs + blockIdx.y] = pow2f(-row_shift(m));
-    }
-}
 
 __device__ __forceinline__ void mma_16816(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
                                           unsigned b0, unsigned b1) {
@@ -57,148 +38,166 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], unsigned a0, unsigned a
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-static const int kTcWarps = 4;
+// c = A B: the first MMA of a sum
+__device__ __forceinline__ void mma_16816_first(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
+                                                unsigned b0, unsigned b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%10, %10, %10, %10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
 
-// NR right-hand sides, B steps of a launch.  Rows in shared memory: row q of the item holds the slip
-// rates of step n + B - 1 - k0 - q, [q][hi, lo][right-hand side][32 sources]; 8 consecutive rows are the
-// columns of one MMA tile, so window slice k takes the tiles from row k - k0 on, B NR / 4 of them
-// (tile = one step of 8 right-hand sides' hi or lo, of 4 with both, 2 steps of 2).
+// NR right-hand sides, B steps of a launch (1 or 16).  Rows in shared memory: row q of the item holds the slip
+// rates of step n + S - 1 - k0 - q, S the steps rounded up to whole tiles, [q][part][right-hand side][32 sources] with
+// the parts hi, lo (one right-hand side: hi, lo, rest, zero); 8 consecutive rows are the columns of one MMA
+// tile, so window slice k takes the tiles from row k - k0 on (tile = one step of 8 right-hand sides' hi or
+// lo, of 4 with both, 2 steps of 2 or of one with its four parts).
+//
+// Warps take 16 receivers and a share of the tiles each, and all slices of the item: the item's sums stay in
+// the accumulators and are written straight out, and 16 steps of 8 right-hand sides take one pass over the
+// coefficients.  With a share of the slices per warp the sums of the four warps met in shared memory and FP64
+// at the end of every item, and two passes were needed: eight right-hand sides, N = 6000, 3.86 -> 3.23 ms per
+// 16 steps (near field 67 us a step); four, N = 2500, 1.69 -> 1.35 ms per 32.  One right-hand side was FP32 multiply-adds on the CUDA cores
+// (near_block_kernel): planar N = 1601, 502 -> 461 us per 32 steps.  Bound by latency and issue slots, not by
+// the tensor pipe: a slice is two 16-byte loads, then two (four) dependent MMAs and four FMAs a tile.
 template <int NR, int B>
 struct TcCfg {
-    static_assert((NR == 2 && B % 2 == 0) || NR == 4 || NR == 8, "whole tiles");
-    static constexpr int C = 2 * NR;                        // columns of one row q
-    static constexpr int tiles = NR == 8 ? B : B * NR / 4;  // accumulator tiles (hi and lo of 8 share one)
-    static constexpr int rows(int chunk) { return chunk + B - 1; }
+    static constexpr int C = NR == 1 ? 4 : 2 * NR;            // columns of one row q
+    static constexpr int per = NR <= 2 ? 8 / C : 1;           // steps of one tile
+    static constexpr int S = B < per ? per : B;
+    static constexpr int tiles = S / per;                     // accumulator tiles (hi and lo of 8 share one)
+    static constexpr int warps = B == 1 ? 2 : 4;
+    static constexpr int share = B == 1 ? 1 : tiles / 2;      // tiles of a warp at most
+    static constexpr int rows(int chunk) { return chunk + S - 1; }
     static constexpr size_t row_bytes(int chunk) { return (size_t)rows(chunk) * C * 64; }
-    // rows and their scales; afterwards the warps' sums
-    static constexpr size_t smem(int chunk) {
-        const size_t a = row_bytes(chunk) + (size_t)rows(chunk) * C * 4, r = (size_t)kTcWarps * B * NR * 32 * 4;
-        return a > r ? a : r;
-    }
+    // rows and their scales
+    static constexpr size_t smem(int chunk) { return row_bytes(chunk) + (size_t)rows(chunk) * C * 4; }
 };
 
 template <int NR, int B>
-__global__ void __launch_bounds__(32 * kTcWarps, 3) tc_block_kernel(StepArgs<float> a) {
+__global__ void __launch_bounds__(32 * TcCfg<NR, B>::warps, B == 1 ? 8 : 4) tc_block_kernel(StepArgs<float> a, int chunk) {
     using Cf = TcCfg<NR, B>;
-    constexpr int C = Cf::C;
+    constexpr int C = Cf::C, S = Cf::S, NW = Cf::warps, T = Cf::share;
     extern __shared__ __align__(16) unsigned char tc_smem[];
     const NearTask tk = a.tasks[blockIdx.x];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n = step_index(a), nb = a.nb, nr = tk.nr, ns = tk.ns;
     const int nk = tk.k0 < n + nb ? tk.k1 - tk.k0 : 0;   // (0: the item's window lies before the march)
-    const int nrow = nk ? nk + B - 1 : 0;
+    const int nrow = nk ? nk + S - 1 : 0;
     __half* rows = (__half*)tc_smem;
-    float* scl = (float*)(tc_smem + Cf::row_bytes(nk > 0 ? nk : 1));
+    float* scl = (float*)(tc_smem + Cf::row_bytes(chunk));
     {
-        const int top = n + B - 1 - tk.k0, hend = hist_end(a, n), stop = wrap(top, a.WD);
-        const float* ring = a.Dring32 + tk.s0 + (lane < ns ? lane : 0);
-        // (the loads of kAhead rows in flight at a time: a row is a dependent pair of loads otherwise, and
-        // the staging, not the MMAs, bounded the kernel)
-        constexpr int kAhead = 8;
-        for (int u0 = warp * kAhead; u0 < nrow * NR; u0 += kTcWarps * kAhead) {
-            float x[kAhead], sc[kAhead];
+        const int top = n + S - 1 - tk.k0, hend = hist_end(a, n), stop = wrap(top, a.WD);
+        // warps over right-hand sides, then over rows, kAhead of them in flight (row by row the staging, not the
+        // MMAs, bounded the kernel)
+        constexpr int kAhead = 8, RW = NR < NW ? NR : NW, QW = NW / RW;
+        const bool src = lane < ns;
+        for (int r = warp % RW; r < NR; r += RW) {
+            const float* ring = a.Dring32 + r * a.rs_D + tk.s0 + (src ? lane : 0);
+            for (int q0 = warp / RW * kAhead; q0 < nrow; q0 += QW * kAhead) {
+                float x[kAhead];
 #pragma unroll
-            for (int i = 0; i < kAhead; ++i) {
-                const int u = u0 + i, q = u / NR, r = u % NR, t = top - q;
-                const bool ok = u < nrow * NR && t >= 0 && t < hend;
-                int slot = stop - q;              // nrow <= WD: one wrap at most
-                slot += slot < 0 ? a.WD : 0;
-                x[i] = ok && lane < ns ? ring[r * a.rs_D + (size_t)slot * a.N] : 0.f;
-                sc[i] = ok ? a.Dscale[(size_t)slot * NR + r] : 0.f;
-            }
+                for (int i = 0; i < kAhead; ++i) {
+                    const int t = top - q0 - i;
+                    int slot = stop - q0 - i;              // nrow <= WD: one wrap at most
+                    slot += slot < 0 ? a.WD : 0;
+                    const bool ok = q0 + i < nrow && t >= 0 && t < hend;
+                    x[i] = ok && src ? ring[(size_t)slot * a.N] : 0.f;
+                }
 #pragma unroll
-            for (int i = 0; i < kAhead; ++i) {
-                const int u = u0 + i, q = u / NR, r = u % NR;
-                if (u >= nrow * NR) break;
-                // 2^sh from 2^-sh: the exponents add up to that of 1
-                const float y = x[i] * (sc[i] > 0.f ? __uint_as_float((254u << 23) - __float_as_uint(sc[i])) : 0.f);
-                const __half hi = __float2half_rn(y);
-                rows[(size_t)(q * C + r) * 32 + lane] = hi;
-                rows[(size_t)(q * C + NR + r) * 32 + lane] = __float2half_rn(y - __half2float(hi));
-                if (lane == 0) scl[q * C + r] = scl[q * C + NR + r] = sc[i];
+                for (int i = 0; i < kAhead; ++i) {
+                    if (q0 + i >= nrow) break;
+                    const int sh = row_shift(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(x[i]))));
+                    const float y = x[i] * pow2f(sh);
+                    const __half hi = __float2half_rn(y);
+                    const float y1 = fabsf(y) <= 65504.f ? y - __half2float(hi) : 0.f;   // (an infinity has no rest)
+                    const __half lo = __float2half_rn(y1);
+                    __half* row = rows + (size_t)((q0 + i) * C + r) * 32 + lane;
+                    row[0] = hi;
+                    row[NR * 32] = lo;
+                    if constexpr (NR == 1) {
+                        row[64] = __float2half_rn(y1 - __half2float(lo));
+                        row[96] = __float2half_rn(0.f);
+                    }
+                    if (lane < C / NR) scl[(q0 + i) * C + lane * NR + r] = pow2f(-sh);
+                }
             }
         }
     }
     __syncthreads();
+    // this warp's receivers 16 mt ... 16 mt + 15 and tiles i0 ... i0 + nt - 1 (leaves of at most 16 receivers
+    // have one set of receivers: a quarter of the tiles per warp; one step: the second warp has nothing to do)
+    const bool two = nr > 16;
+    const int mt = two ? warp & 1 : 0;
+    const int nt = B == 1 ? (two || warp == 0 ? 1 : 0) : two ? T : T / 2;
+    const int i0 = B == 1 ? 0 : (two ? warp >> 1 : warp) * nt;
+    if (!nt) return;
     const int g = lane >> 2, t = lane & 3;
-    // the 16-byte vectors (sources 8 t ... 8 t + 7) of receivers g, g + 8, g + 16, g + 24
-    const __half* base = (const __half*)a.tensor + tk.off;
+    // the 16-byte vectors (sources 8 t ... 8 t + 7) of receivers g and g + 8 of the set
+    const __half* base = (const __half*)a.tensor + tk.off + ((size_t)t * nr + 16 * mt + g) * 8;
     const bool in = FDPH_IDX(tk.off + (long long)nk * tk.sl <= a.len_tensor, a.err) && 8 * t < ns;
-    auto load = [&](int k, uint4 (&x)[4]) {
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int i = g + 8 * m;
-            x[m] = in && k < nk && i < nr ? __ldcs((const uint4*)(base + (size_t)k * tk.sl + ((size_t)t * nr + i) * 8))
-                                          : make_uint4(0, 0, 0, 0);
-        }
-    };
-    float acc[Cf::tiles][2][4];
-#pragma unroll
-    for (int i = 0; i < Cf::tiles; ++i)
+    auto load = [&](int k, uint4 (&x)[2]) {
 #pragma unroll
         for (int m = 0; m < 2; ++m)
+            x[m] = in && k < nk && 16 * mt + g + 8 * m < nr ? __ldcs((const uint4*)(base + (size_t)k * tk.sl + 64 * m))
+                                                             : make_uint4(0, 0, 0, 0);
+    };
+    float acc[T][4];
 #pragma unroll
-            for (int f = 0; f < 4; ++f) acc[i][m][f] = 0.f;
-    uint4 x[4], xn[4];
-    load(warp, xn);
-    for (int k = warp; k < nk; k += kTcWarps) {
+    for (int i = 0; i < T; ++i)
 #pragma unroll
-        for (int m = 0; m < 4; ++m) x[m] = xn[m];
-        load(k + kTcWarps, xn);
-        const __half* rk = rows + ((size_t)k * C + g) * 32 + 8 * t;
-        const float* sk = scl + k * C + 2 * t;
+        for (int f = 0; f < 4; ++f) acc[i][f] = 0.f;
+    constexpr int D = 2;   // slices in flight
+    uint4 xn[D][2];
 #pragma unroll
-        for (int i = 0; i < Cf::tiles; ++i) {
-            float c[2][4];
+    for (int d = 0; d < D; ++d) load(d, xn[d]);
+    constexpr int parts = NR == 8 ? 2 : 1;   // (8 right-hand sides: the hi tile, then the lo tile)
+    const __half* rk = rows + ((size_t)i0 * parts * 8 + g) * 32 + 8 * t;
+    const float* sk = scl + i0 * parts * 8 + 2 * t;
+    for (int k = 0; k < nk; ++k, rk += C * 32, sk += C) {
+        const uint4 x0 = xn[0][0], x1 = xn[0][1];
 #pragma unroll
-            for (int m = 0; m < 2; ++m)
+        for (int d = 0; d + 1 < D; ++d) {
+            xn[d][0] = xn[d + 1][0];
+            xn[d][1] = xn[d + 1][1];
+        }
+        load(k + D, xn[D - 1]);
 #pragma unroll
-                for (int f = 0; f < 4; ++f) c[m][f] = 0.f;
-            constexpr int parts = NR == 8 ? 2 : 1;   // (8 right-hand sides: the hi tile, then the lo tile)
+        for (int i = 0; i < T; ++i) {
+            if (i >= nt) break;   // (warp-uniform)
+            float c[4];
 #pragma unroll
             for (int h = 0; h < parts; ++h) {
                 const uint4 b = *(const uint4*)(rk + (size_t)(i * parts + h) * 8 * 32);
-#pragma unroll
-                for (int m = 0; m < 2; ++m) mma_16816(c[m], x[2 * m].x, x[2 * m + 1].x, x[2 * m].y, x[2 * m + 1].y, b.x, b.y);
-#pragma unroll
-                for (int m = 0; m < 2; ++m) mma_16816(c[m], x[2 * m].z, x[2 * m + 1].z, x[2 * m].w, x[2 * m + 1].w, b.z, b.w);
+                if (h == 0) mma_16816_first(c, x0.x, x1.x, x0.y, x1.y, b.x, b.y);
+                else mma_16816(c, x0.x, x1.x, x0.y, x1.y, b.x, b.y);
+                mma_16816(c, x0.z, x1.z, x0.w, x1.w, b.z, b.w);
             }
             const float2 s = *(const float2*)(sk + i * parts * 8);
-#pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                acc[i][m][0] = fmaf(c[m][0], s.x, acc[i][m][0]);
-                acc[i][m][1] = fmaf(c[m][1], s.y, acc[i][m][1]);
-                acc[i][m][2] = fmaf(c[m][2], s.x, acc[i][m][2]);
-                acc[i][m][3] = fmaf(c[m][3], s.y, acc[i][m][3]);
-            }
+            acc[i][0] = fmaf(c[0], s.x, acc[i][0]);
+            acc[i][1] = fmaf(c[1], s.y, acc[i][1]);
+            acc[i][2] = fmaf(c[2], s.x, acc[i][2]);
+            acc[i][3] = fmaf(c[3], s.y, acc[i][3]);
         }
     }
-    __syncthreads();   // the rows have been read: their place takes the warps' sums
-    // red[warp][step][right-hand side][receiver]
-    float* red = (float*)tc_smem + (size_t)warp * B * NR * 32;
-#pragma unroll
-    for (int i = 0; i < Cf::tiles; ++i)
-#pragma unroll
-        for (int m = 0; m < 2; ++m)
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                float v = acc[i][m][f];
-                if constexpr (NR == 4) v += __shfl_xor_sync(0xffffffffu, v, 2);   // hi + lo
-                if constexpr (NR == 2) v += __shfl_xor_sync(0xffffffffu, v, 1);
-                const int col = 2 * t + (f & 1);          // column of the tile
-                const int q = NR == 2 ? 2 * i + (col >> 2) : i, r = col % NR;
-                const bool mine = NR == 8 || (NR == 4 ? col < 4 : !(col & 2));
-                if (mine) red[((B - 1 - q) * NR + r) * 32 + 16 * m + g + 8 * (f >> 1)] = v;
-            }
-    __syncthreads();
-    if (!FDPH_IDX((long long)tk.item * 32 + 32 <= a.cap_partial, a.err)) return;
+    const bool fits = FDPH_IDX((long long)tk.item * 32 + 32 <= a.cap_partial, a.err);
     const float ks = a.kinv;   // the window's storage scale (a power of two)
-    for (int u = threadIdx.x; u < nb * NR * 32; u += 32 * kTcWarps) {
-        const int i = u & 31, r = (u >> 5) % NR, b = (u >> 5) / NR;
-        const float* v = (const float*)tc_smem + (size_t)(b * NR + r) * 32 + i;
-        double s = wide(v[0] * ks);
+    double* out = a.partial + (size_t)tk.item * 32 + 16 * mt;
 #pragma unroll
-        for (int w = 1; w < kTcWarps; ++w) s += wide(v[(size_t)w * B * NR * 32] * ks);
-        if (i < nr) a.partial[r * a.rs_partial + b * a.cap_partial + (size_t)tk.item * 32 + i] = s;
+    for (int i = 0; i < T; ++i) {
+        if (i >= nt) break;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            float v = acc[i][f];
+            if constexpr (NR == 4) v += __shfl_xor_sync(0xffffffffu, v, 2);   // hi + lo
+            if constexpr (NR == 1) v += acc[i][f ^ 1];                         // hi + lo, rest + 0
+            if constexpr (NR <= 2) v += __shfl_xor_sync(0xffffffffu, v, 1);
+            const int col = 2 * t + (f & 1);          // column of the tile
+            const int q = Cf::per * (i0 + i) + (NR <= 2 ? col >> 2 : 0), r = col % NR, b = S - 1 - q;
+            const bool mine = NR == 8 || (NR == 4 ? col < 4 : NR == 2 ? !(col & 2) : !(col & 3));
+            const int row = g + 8 * (f >> 1);
+            if (mine && fits && b < nb && 16 * mt + row < nr) out[r * a.rs_partial + b * a.cap_partial + row] = wide(v * ks);
+        }
     }
 }
