@@ -361,8 +361,8 @@ def run_serving(args):
 
 def batch_vs_streams(fdph, serving, count=16, chunk=64, rounds=4):
     """GPU stepping of `count` resident rupture scenarios (plans built beforehand, N log-uniform
-    in [256, 2048], curved, CFL 1/2, FP32): `rounds` chunks of `chunk` steps as one batch (one
-    near-field launch per step for all) against each scenario's own step graph on its own
+    in [256, 2048], curved, CFL 1/2, FP32): `rounds` chunks of `chunk` steps as one batch
+    (one call) against each scenario's own calls, both with each scenario's graphs on its own
     stream.  Device-side time of the whole chunk round, host clock around synchronisations."""
     import torch
     reqs = serving.poisson_requests(count, rate=8.0, seed=9, n_min=256, n_max=2048, cfls=(0.5,))

@@ -1,32 +1,14 @@
 // fdph.cu -- device side of the FDP=H time step and the C ABI (include/fdph.h).
 //
-// One time step n (Eq. 4 evaluated through the plan's operator) runs these kernels (captured
-// as one CUDA graph: FIR + scatter and transient + Eq. 39 on two side streams, concurrently with
-// the near field, all joined before gather; several right-hand sides go through one launch, the
-// far-field kernels taking all of them in a thread or warp):
-//   push     D_n -> slip-rate ring (internal order); cumulative slip C_j(n) = sum_{s<=n} D_j,s
-//            with a compensated (Kahan) FP64 sum, -> cumulative-slip ring; with the tensor-core
-//            near field (FP16 window, several right-hand sides) also the ring row's scaled FP16
-//            (hi, lo) copy (tc_rows)
-//   fir      Domain F, formula 1 (Eq. 32): Dhat_j = sum_{m < Dm_j} h_{j,m} D_{j,n-m}, per F block
-//            and source (fir), or per source for all its F blocks (sfir), in the factor type
-//   scatter  formula 2 (Eq. 42): Tbar'_l[n + delay_j] += g_{l,j} u_j for every run of sources
-//            (rings are stored [slot][rank] so that one receiver's ranks share a sector)
-//            with equal delay (no atomics: one writer per ring slot); u = Dhat (Domain F),
-//            dt * C (Domain S, App. B.1 written on the cumulative slip), D (transient);
-//            the ring is the shift operator M of Eq. 40 as a base-pointer increment
-//   trconv   transient (App. B.3): Z_l(n - min dm) = sum_{m < Dm_tr} h^tr_m Y_l(n - min dm - m)
-//   near     inadmissible leaves (App. E): sum_{k < W} K_{ij,k} D_{j,n-k} + Kstat_ij dt C_j(n-W),
-//            per (leaf, chunk of k) work item into a partial-sum slot
-//   far_eval + far_sum  formula 3 (Eq. 39): Tfar_i = sum_{blocks} sum_l f_{l,i} Tbar'_l[n - dm_i]
-//            (far-field branch)
-//   gather   T_i = Tfar_i + the receiver's near partials, written in the caller's element order
-// Causality (min(dm + delay) >= 1, checked at plan time) guarantees that the ring slots read
-// at step n were completed by steps < n and that the slots written at step n are not read.
-// A rupture step (Sec. 6.2) predicts with D_n = 0, solves the friction law per element and
-// then commits D_n; a batch of plans runs each of these kernels as one launch over all plans.
-#include <cuda.h>
-#include <cudaTypedefs.h>
+// Steps run in blocks of up to 16 (step.cuh); the kernels of a block are captured as one CUDA graph: FIR +
+// scatter and transient + Eq. 39 on two side streams, beside the near field, all joined before the gather.
+// Causality (min(dm + delay) >= 1, checked at plan time) guarantees that the ring slots read at step n were
+// completed by steps < n and that the slots written at step n are not read; where min(dm + delay) is less
+// than the block's length, Eq. 39 follows the scatter.  The near field runs on the CUDA cores (FP32, step.cuh)
+// or on the tensor cores (FP16 windows, tensor.cuh; FP64 by exact products, fixed.cuh).  Several right-hand
+// sides go through one launch.  A rupture block (Sec. 6.2) takes what the slip rates before the block do to
+// all its steps at once, then step by step its own part, the friction law and the push, then commits the
+// block.  A batch runs its plans on their own streams.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -324,7 +306,7 @@ struct fdph_plan_s {
     void* dhat = nullptr;
     size_t state_bytes = 0;
     // host staging for fdph_step_host
-    double *hD = nullptr, *hT = nullptr, *dD = nullptr, *dT = nullptr;
+    double *dD = nullptr, *dT = nullptr;
     // per-kernel event timing
     bool prof = false;
     struct ProfEvent {
@@ -1034,7 +1016,7 @@ static int build_schedule(fdph_plan_t P) {
 
 // Near-field build in two phases around the host factorisation of the admissible blocks, which
 // it does not need: build_near_begin (windows, exact tensors, tail projections launched on the
-// device) and build_near_finish (tail fits on the host, upload, persistent schedule).
+// device) and build_near_finish (tail fits on the host, upload, schedule).
 struct NearBuild {
     std::vector<NearDev> tl;        // leaves with an exponential tail
     std::vector<long long> tp0;     // their first pair
@@ -1442,7 +1424,7 @@ static void fill_stats(fdph_plan_t P) {
 }
 
 // Near-field work items of `chunk` kernel steps (1..kChunk): new items, partial slots and
-// persistent schedule; the stored coefficients do not move.  Cached step graphs refer to the old
+// schedule; the stored coefficients do not move.  Cached step graphs refer to the old
 // schedule and are dropped.
 template <class T, class H>
 static int set_chunk(fdph_plan_t P, int chunk) {
@@ -1820,7 +1802,7 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
         const SubBlock& b = hp.sbs[q];
         const int LH = b.maxdelay - b.mindelay + 1;
         sd[q] = {b.kind, b.rank, b.r0, b.nr, b.s0, b.ns, b.L, b.LZ, b.taps, b.maxdelay, b.mindm, b.run0,
-                 b.soe, b.ident, b.e0, LH, (long long)b.f, (long long)b.g, (long long)b.h, (long long)b.ring, (long long)b.zring,
+                 b.soe, b.ident, LH, (long long)b.f, (long long)b.g, (long long)b.h, (long long)b.ring, (long long)b.zring,
                  (long long)b.dhat, (long long)b.delay, (long long)b.dm, (long long)b.ustate, (long long)b.trc,
                  (long long)b.phi, 0, b.mindelay, b.qn, (long long)b.qb};
     }

@@ -429,7 +429,6 @@ int build_host_far(const Elements& el, const PlanInputs& in, HostPlan& hp) {
             sb.maxdelay = *std::max_element(dl.begin(), dl.end());
             sb.mindelay = *std::min_element(dl.begin(), dl.end());
             sb.mindm = mindm;
-            sb.maxdm = maxdm;
             sb.taps = taps;
             sb.f = append(hp.fac, lr.F.data(), lr.F.size());
             sb.g = append(hp.fac, lr.G.data(), lr.G.size());
@@ -451,8 +450,6 @@ int build_host_far(const Elements& el, const PlanInputs& in, HostPlan& hp) {
             sb.soe = soe;
             sb.trc = trc ? append(hp.trcoef, trc->data(), trc->size()) : 0;
             sb.ident = lr.exact ? (lr.m <= lr.n ? 1 : 2) : 0;
-            sb.e0 = (int32_t)hp.far_nent;
-            hp.far_nent += o.nr;
             sb.ustate = hp.ustate_len;   // [rank][soe + qn]: exponential-tail states, then running sums
             hp.ustate_len += (int64_t)sb.rank * (soe + sb.qn);
             if (kind == SB_TR) {
@@ -542,16 +539,6 @@ int build_host_far(const Elements& el, const PlanInputs& in, HostPlan& hp) {
         for (size_t q = 0; q < hp.fir_sb.size(); ++q) {
             const int p = hp.sbs[hp.fir_sb[q]].s0 + hp.fir_j[q];
             hp.sfir_q[fill[p]++] = (int32_t)q;
-        }
-    }
-    // block-major list of the same entries; recv[p] was filled in increasing block order, so the
-    // k-th visit of receiver p is its k-th CSR slot
-    std::vector<int32_t> cnt(n, 0);
-    for (int id = 0; id < (int)hp.sbs.size(); ++id) {
-        const SubBlock& sb = hp.sbs[id];
-        for (int il = 0; il < sb.nr; ++il) {
-            const int p = sb.r0 + il;
-            hp.e_pos.push_back(hp.g_ptr[p] + cnt[p]++);
         }
     }
     return 0;

@@ -21,7 +21,7 @@ struct SubBlock {
                        // slots of it beyond what one step needs
     int32_t LZ;        // TR: length of the convolved ring Z (with the same room)
     int32_t taps;      // F: waveform taps (max Dm of the leaf); TR: Dm_tr
-    int32_t maxdelay, mindelay, mindm, maxdm;
+    int32_t maxdelay, mindelay, mindm;
     int64_t f, g, h;   // offsets into the factor array (f: nr x rank, g: ns x rank, h: taps x ns or taps)
     int64_t ring, zring, dhat;   // offsets into state arrays
     int64_t delay, dm; // offsets into the int array (delay[ns], dm[nr])
@@ -32,7 +32,6 @@ struct SubBlock {
     int64_t phi;       // offset of the receivers' sub-step delays in HostPlan::phis (interp only)
     int32_t ident;     // block kept exact: 1 = F is the identity (rank nr), 2 = G is the identity
                        // (rank ns), 0 = low-rank factors
-    int32_t e0;        // index of the block's first (block, receiver) entry in block-major order
     int32_t qn;        // TR with eps_q > 0: quantized ranges of the taps (h then holds their qn values)
     int64_t qb;        // TR: offset of the qn + 1 range bounds in the int array
 };
@@ -54,8 +53,7 @@ struct NearLeaf {
     int64_t vstate;              // offset of the [Q][ns] recursive tail states
 };
 
-// A near-field work item: window slices [k0, k1) of a leaf (kind 0), or its aux slices (kind 1).
-// a work item: window slices [k0, k1) of a leaf (kind 0), or its aux slices [k0, k1) (kind 1:
+// A near-field work item: window slices [k0, k1) of a leaf (kind 0), or its aux slices [k0, k1) (kind 1:
 // slice 0 the static tile, slice 1 + q the exponential-tail coefficients of term q)
 struct NearItem {
     int32_t leaf, k0, k1, kind;
@@ -80,7 +78,6 @@ struct HostPlan {
     std::vector<int32_t> sfir_ptr, sfir_q, sfir_tmax; // FIR tasks by source element, longest taps
     std::vector<int32_t> tr_sb, tr_l;                // transient convolution tasks
     std::vector<int32_t> g_ptr, g_sb, g_il;          // gather CSR (receiver-major)
-    std::vector<int32_t> e_pos;                      // CSR slot of each entry, block-major order
     int64_t ring_len = 0, zring_len = 0, dhat_len = 0, ustate_len = 0;
     int soe = 0;                                     // exponential-tail terms (0: paper's cut)
     std::vector<double> rho;                         // their decay factors
@@ -99,7 +96,6 @@ struct HostPlan {
     int n_exact[3] = {0, 0, 0};                          // per SubKind: sub-blocks kept exact
     int n_aca = 0;                                       // sub-blocks from cross approximation
     int64_t far_entries = 0;
-    int64_t far_nent = 0;                            // (block, receiver) entries
 };
 
 // Everything except the near-field windows (which need the device). Returns status.

@@ -47,7 +47,7 @@ __device__ __forceinline__ bool fdph_idx_check(bool ok, int* err) {
 #endif
 
 struct SbDev {
-    int kind, rank, r0, nr, s0, ns, L, LZ, taps, maxdelay, mindm, run0, soe, ident, e0, LH;
+    int kind, rank, r0, nr, s0, ns, L, LZ, taps, maxdelay, mindm, run0, soe, ident, LH;
     long long f, g, h, ring, zring, dhat, delay, dm, ustate, trc, phi;
     long long uhist;    // delayed-history form: [LH][ns] source values u_j of the last LH steps
     int mindelay, qn;   // qn: quantized ranges of a transient's taps (0: exact taps)

@@ -361,8 +361,8 @@ def plain_step_noalloc(K, n, W, D_hist, hist_len, step, T, stream=None):
 
 
 class Batch:
-    """Plans stepped together with one near-field launch per step (fdph_batch_create); the
-    plans must outlive the batch."""
+    """Plans stepped together, each on its own stream (fdph_batch_create); the plans must outlive
+    the batch."""
 
     def __init__(self, plans):
         L = lib()

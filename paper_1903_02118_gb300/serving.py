@@ -4,8 +4,8 @@ Requests (fault geometry, size N, CFL, friction heterogeneity) arrive over time.
 admitted as soon as its device footprint (plan operator + time-stepping state + outputs) fits
 the HBM budget and a slot is free; admitted scenarios stay resident and all of them advance
 together, each iteration moving every live scenario forward by `chunk` time steps: the
-scenarios with a full chunk ahead as one batch (fdph_batch_rupture_run: every kernel of a step
-is one launch over all of them), the others (a last, shorter chunk) with their own step graphs
+scenarios with a full chunk ahead as one batch (fdph_batch_rupture_run: every plan's blocks of
+steps on the plan's own stream), the others (a last, shorter chunk) with their own step graphs
 on their own CUDA streams.  A finished scenario releases its memory at once and the next
 waiting request takes its place.  Per request the loop records queueing, plan and run times and
 the time to solution (arrival to last step on the device).
