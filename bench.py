@@ -55,10 +55,10 @@ METRIC_REL_ERR = 1e-4      # the metric's accuracy condition (relative error vs 
 # near-field coefficient: the near bytes scale with the stored coefficients, so a full launch's
 # traffic is this figure times the plan's coefficients.  Reported only while the near-field
 # kernel's source (near_kernel_source_hash) is the one that was captured.
-NEAR_NCU = {"source_sha256": "c08939cd1e5992346e6387f5e23eac9888631ec999bc2fb830ab141666903a18",
-            "dram_bytes_per_coefficient": 4.1471, "precision": 1, "nrhs": 1,
-            "capture": "profiles/near_kernel_curved_n2048_m1024_fp32_soe16.md (curved N = 2048, M = 1024, FP32, "
-                       "Q = 16, two steady-state launches)"}
+NEAR_NCU = {"source_sha256": "b8e0626781aed8c333d157ee8d30181af24daae8ddebe2f261d6f2d908deb1aa",
+            "dram_bytes_per_coefficient": 1.453, "precision": 1, "nrhs": 1,
+            "capture": "profiles/block_kernels_curved_n2048_m1024.md (curved N = 2048, M = 1024, FP32, "
+                       "Q = 16, one launch of 16 steps)"}
 
 
 def near_kernel_source_hash():
@@ -424,7 +424,8 @@ def time_steps(plan, stream, Dd, Td, n_from, K):
 
 def near_roofline(plan, st, Dd, Td, n_from, K, hbm_peak):
     """Per-kernel CUDA-event times over K steps from n_from (profiling on) and the near-field
-    kernel's achieved bandwidth: algorithmic near bytes per launch / its mean launch time."""
+    kernel's achieved bandwidth: algorithmic near bytes / time, the operator read once per launch of
+    up to 16 steps."""
     plan.reset()
     if n_from:
         plan.run(n_from, Dd, Td)
@@ -434,7 +435,7 @@ def near_roofline(plan, st, Dd, Td, n_from, K, hbm_peak):
     kt = plan.kernel_times()
     plan.set_profiling(False)
     near_ms = kt["near"][0] / max(kt["near"][1], 1)
-    achieved = st["near_bytes_per_step"] / (near_ms * 1e-3) / 1e9
+    achieved = st["near_bytes_per_step"] * -(-K // 16) / K / (near_ms * 1e-3) / 1e9
     return kt, {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                 "kernel": "near_block_kernel", "kernel_ms": {k: v[0] / max(v[1], 1) for k, v in kt.items()}}
 
@@ -641,7 +642,7 @@ def run_fdph(args, cfg):
     ok_case = same and prec == NEAR_NCU["precision"] and R == NEAR_NCU["nrhs"] and cfg.get("soe")
     roofline["traffic"] = NEAR_NCU["dram_bytes_per_coefficient"] * st["near_entries"] if ok_case else None
     roofline["traffic_note"] = ("ncu dram read+write per stored coefficient of " + NEAR_NCU["capture"] +
-                                ", times this plan's stored coefficients") if ok_case \
+                                ", times this plan's stored coefficients: bytes of a launch of 16 steps") if ok_case \
         else "no ncu capture of this kernel version / precision / right-hand sides"
 
     # end to end through the C ABI with host buffers (page-locked): fdph_run_host copies every

@@ -592,8 +592,8 @@ static void launch_near_aux(fdph_plan_t P, StepArgs<T> a, cudaStream_t s) {
         if (P->precision != FDPH_FP16 || !P->n_aux) return;
         a.tasks += P->n_win;
         a.n_items = P->n_aux;
-        if (a.nb == 1) launch_near_items<T, __half, 1>(a, P->chunk, s);
-        else launch_near_items<T, __half, kBlk>(a, P->chunk, s);
+        if (a.nb == 1) launch_near_items<T, float, 1>(a, P->chunk, s);
+        else launch_near_items<T, float, kBlk>(a, P->chunk, s);
     }
 }
 
@@ -1002,10 +1002,10 @@ static int build_schedule(fdph_plan_t P) {
         FDPH_CUDA(cudaFuncSetAttribute(fixed_block_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FxCfg<1>::smem(kChunk)));
         FDPH_CUDA(cudaFuncSetAttribute(fixed_block_kernel<kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FxCfg<kBlk>::smem(kChunk)));
     } else {
-        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, H, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)NearCfg<H, 1>::warp_bytes(2 * kChunk) * kNearWarps));
-        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, H, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)NearCfg<H, kBlk>::warp_bytes(2 * kChunk) * kNearWarps));
+        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, float, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)NearCfg<float, 1>::warp_bytes(2 * kChunk) * kNearWarps));
+        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, float, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)NearCfg<float, kBlk>::warp_bytes(2 * kChunk) * kNearWarps));
     }
     P->sched_version += 1;
     int rc;

@@ -674,7 +674,7 @@ __global__ void gather_kernel(StepArgs<T> a0) {
     }
 }
 
-// ---- near field (App. E) on the CUDA cores (FP32 and FP16 plans; FP64: fixed.cuh)
+// ---- near field (App. E) on the CUDA cores (FP32 items; FP16 windows: tensor.cuh, FP64 plans: fixed.cuh)
 
 // Near-field storage: window slices in H; aux slices (static tile, tail coefficients) in the aux
 // type (FP32 when the window is FP16: the static term multiplies the cumulative slip, so its
@@ -819,10 +819,7 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
                 for (int jb = 0; jb < nbk; ++jb) {
                     R x[G][V];
 #pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        if constexpr (sizeof(H) == 2) unpack(xn[g], x[g], __half());
-                        else unpack(xn[g], x[g], R());
-                    }
+                    for (int g = 0; g < G; ++g) unpack(xn[g], x[g], R());
                     const bool wrapj = jb + 1 == nbk;
                     load(wrapj ? gr + ngrp : gr, wrapj ? 0 : jb + 1, xn);
                     {
