@@ -234,7 +234,7 @@ typedef struct fdph_friction {
     int32_t law;          /* 0: linear slip weakening, 1: exponential slip weakening */
 } fdph_friction;
 
-/* Attach a friction law to a plan (copies tau0; zero slip).  Errors: FDPH_E_ARG, FDPH_E_OOM,
+/* Attach a friction law to a plan, or replace the one it has (copies tau0; zero slip).  Errors: FDPH_E_ARG, FDPH_E_OOM,
  * FDPH_E_CUDA, FDPH_E_STATE (instantaneous term not local: cs dt > min element length / 2). */
 int fdph_rupture_init(fdph_plan_t plan, const fdph_friction* friction);
 

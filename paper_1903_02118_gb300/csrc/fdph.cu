@@ -2356,8 +2356,12 @@ int fdph_rupture_init(fdph_plan_t P, const fdph_friction* f) {
     if (rc0) return rc0;
     if (!P->rupture) {
         double *tau0 = nullptr, *kk = nullptr, *slip = nullptr;
+        FrictionLaw* law = nullptr;
         int rc;
-        if ((rc = dalloc(P, &tau0, P->N)) || (rc = dalloc(P, &kk, P->N)) || (rc = dalloc(P, &slip, P->N))) return rc;
+        if ((rc = dalloc(P, &tau0, P->N)) || (rc = dalloc(P, &kk, P->N)) || (rc = dalloc(P, &slip, P->N)) ||
+            (rc = dalloc(P, &law, 1)))
+            return rc;
+        P->fr.law = law;
         P->fr.tau0 = tau0;
         P->fr.k0 = kk;
         P->fr.slip = slip;
@@ -2365,14 +2369,11 @@ int fdph_rupture_init(fdph_plan_t P, const fdph_friction* f) {
     // ordered after the caller's work on the plan's stream (tau0 may have been written there)
     FDPH_CUDA(cudaMemcpyAsync((void*)P->fr.tau0, f->tau0, P->N * sizeof(double), cudaMemcpyDeviceToDevice, P->stream));
     FDPH_CUDA(cudaMemcpyAsync((void*)P->fr.k0, k0.data(), P->N * sizeof(double), cudaMemcpyHostToDevice, P->stream));
+    const FrictionLaw law{f->sigma_n, f->mu_s, f->mu_d, f->Dc, f->law};
+    FDPH_CUDA(cudaMemcpyAsync((void*)P->fr.law, &law, sizeof(law), cudaMemcpyHostToDevice, P->stream));
     FDPH_CUDA(cudaMemsetAsync(P->fr.slip, 0, P->N * sizeof(double), P->stream));
     FDPH_CUDA(cudaStreamSynchronize(P->stream));
-    P->fr.sigma_n = f->sigma_n;
-    P->fr.mu_s = f->mu_s;
-    P->fr.mu_d = f->mu_d;
-    P->fr.Dc = f->Dc;
     P->fr.dt = P->dt;
-    P->fr.law = f->law;
     P->rupture = true;
     return FDPH_OK;
 }

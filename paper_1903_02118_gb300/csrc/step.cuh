@@ -939,13 +939,20 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
 
 // ---- rupture (Sec. 6.2)
 
+// Friction law of a plan.  In device memory, like tau0: a captured graph of rupture steps replays the law
+// that fdph_rupture_init last wrote, not the one it was captured with.
+struct FrictionLaw {
+    double sigma_n, mu_s, mu_d, Dc;
+    int law;               // 0: linear slip weakening, 1: exponential (Sec. 6.2)
+};
+
 // Local friction solve (geometry order).
 struct FrictionDev {
+    const FrictionLaw* law;
     const double* tau0;
     const double* k0;      // instantaneous self coefficient K_{ii,0} (< 0)
     double* slip;
-    double sigma_n, mu_s, mu_d, Dc, dt;
-    int law;               // 0: linear slip weakening, 1: exponential (Sec. 6.2)
+    double dt;
 };
 
 // One step of a rupture block.  The traction of step n with D_n = 0 is thist (everything that the
@@ -973,6 +980,7 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
     __shared__ __align__(16) R row[W][2][36];
     __shared__ double red[W][32];
     __shared__ RecLeaf leaves[kRupLeaves];
+    __shared__ FrictionLaw law;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const RecGroup g = a.rec_groups[blockIdx.x];
     const int nf = step_index(a), n = nf + b;
@@ -983,6 +991,7 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
         const int m = min(g.nleaf, kRupLeaves) * words;
         for (int q = threadIdx.x; q < m; q += kRupThreads) ((int4*)leaves)[q] = ((const int4*)(a.rec_leaves + g.leaf0))[q];
     }
+    if (threadIdx.x == 32) law = *f.law;
     // the first warp's element
     const bool mine = warp == 0 && lane < g.nr;
     const int p = g.r0 + lane, e = mine ? a.perm[p] : 0;
@@ -1107,11 +1116,11 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
     const long long off = io_offset(a, nf) + (long long)b * a.io_stride + e;
     const double tau = tau0 + T0;
     double strength;
-    if (f.law == 1) {
-        strength = f.sigma_n * (f.mu_d + (f.mu_s - f.mu_d) * exp(-u / f.Dc));
+    if (law.law == 1) {
+        strength = law.sigma_n * (law.mu_d + (law.mu_s - law.mu_d) * exp(-u / law.Dc));
     } else {
-        const double w = u < f.Dc ? u / f.Dc : 1.0;
-        strength = f.sigma_n * (f.mu_s - (f.mu_s - f.mu_d) * w);
+        const double w = u < law.Dc ? u / law.Dc : 1.0;
+        strength = law.sigma_n * (law.mu_s - (law.mu_s - law.mu_d) * w);
     }
     const double eta = -k0;
     const double d = tau > strength ? (tau - strength) / eta : 0.0;
