@@ -277,8 +277,9 @@ int fdph_commit(fdph_plan_t plan, const double* D_n);
  *   pending), FDPH_E_CUDA.  fdph_autotune on a member plan invalidates the batch (later batch
  *   calls return FDPH_E_STATE; create it again).
  * fdph_batch_run: `steps` steps of every plan; D[p], T[p] (host arrays of device pointers):
- *   plan p's rows, steps * n_p doubles, step-major, as fdph_run.  Asynchronous on the plans'
- *   streams.  Errors as fdph_run for any plan.
+ *   plan p's rows, steps * n_p doubles, step-major, as fdph_run.  Asynchronous; the batch's work starts
+ *   after what is queued on every plan's stream, and every plan's stream is ordered after it.  Errors
+ *   as fdph_run for any plan.
  * fdph_batch_rupture_run: the same for rupture steps (fdph_rupture_init on every plan) with the
  *   outputs of fdph_rupture_run.
  * fdph_batch_synchronize: wait for the batch's plans; reports a device error (as

@@ -1471,13 +1471,28 @@ static int pending_commit(fdph_plan_t P) {
 
 // A set of plans (same device, same precision) stepped together: each plan's blocks run on its own
 // stream, side by side on the GPU.  (One launch per kernel over the work of all plans was measured
-// slower: with a block of steps per launch the launches no longer count, and plans of different
-// sizes need not wait for one another.)
+// slower: with a block of steps per launch the launches no longer count.)  A call starts after the work
+// queued on the streams of all its plans, and they all wait for its end (batch_join), so that a caller
+// may prepare or read the buffers of every plan on the stream of any.
 struct fdph_batch_s {
     int device = 0, precision = 0;
     std::vector<fdph_plan_t> plans;
     std::vector<int> version;            // each plan's near-field schedule at creation
+    cudaStream_t hub = nullptr;          // where the plans' streams meet
+    cudaEvent_t ev_plan = nullptr, ev_hub = nullptr;
 };
+
+// What is queued on any of the plans' streams precedes what is queued on any of them from now on
+static int batch_join(fdph_batch_t B) {
+    if (B->plans.size() < 2) return FDPH_OK;
+    for (fdph_plan_t P : B->plans) {   // (a wait holds the event as it was recorded last: one event does)
+        FDPH_CUDA(cudaEventRecord(B->ev_plan, P->stream));
+        FDPH_CUDA(cudaStreamWaitEvent(B->hub, B->ev_plan, 0));
+    }
+    FDPH_CUDA(cudaEventRecord(B->ev_hub, B->hub));
+    for (fdph_plan_t P : B->plans) FDPH_CUDA(cudaStreamWaitEvent(P->stream, B->ev_hub, 0));
+    return FDPH_OK;
+}
 
 // batch calls: every plan still has the schedule the batch was built on and no pending predict
 static int batch_check(fdph_batch_t B, int steps) {
@@ -2504,6 +2519,14 @@ int fdph_batch_create(const fdph_plan_t* plans, int32_t count, fdph_batch_t* out
     B->precision = plans[0]->precision;
     B->plans.assign(plans, plans + count);
     for (int p = 0; p < count; ++p) B->version.push_back(plans[p]->sched_version);
+    cudaSetDevice(B->device);
+    if (cudaStreamCreateWithFlags(&B->hub, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&B->ev_plan, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&B->ev_hub, cudaEventDisableTiming) != cudaSuccess) {
+        set_error("fdph_batch_create: cudaStreamCreate / cudaEventCreate failed");
+        fdph_batch_destroy(B);
+        return FDPH_E_CUDA;
+    }
     *out = B;
     return FDPH_OK;
 }
@@ -2515,9 +2538,10 @@ int fdph_batch_run(fdph_batch_t B, int32_t steps, const double* const* D, double
     int rc = batch_check(B, steps);
     if (rc || steps == 0) return rc;
     cudaSetDevice(B->device);
-    for (size_t p = 0; p < B->plans.size(); ++p)
-        if ((rc = run_any(B->plans[p], steps, D[p], T[p]))) return rc;
-    return FDPH_OK;
+    if ((rc = batch_join(B))) return rc;
+    for (size_t p = 0; p < B->plans.size() && !rc; ++p) rc = run_any(B->plans[p], steps, D[p], T[p]);
+    const int joined = batch_join(B);   // (after an error too: some plans may have been launched)
+    return rc ? rc : joined;
 }
 
 int fdph_batch_rupture_run(fdph_batch_t B, int32_t steps, double* const* D, double* const* T) {
@@ -2532,12 +2556,13 @@ int fdph_batch_rupture_run(fdph_batch_t B, int32_t steps, double* const* D, doub
     int rc = batch_check(B, steps);
     if (rc || steps == 0) return rc;
     cudaSetDevice(B->device);
-    for (size_t p = 0; p < B->plans.size(); ++p) {
+    if ((rc = batch_join(B))) return rc;
+    for (size_t p = 0; p < B->plans.size() && !rc; ++p) {
         fdph_plan_t P = B->plans[p];
         rc = P->precision != FDPH_FP64 ? rupture_steps<float>(P, steps, D[p], T[p]) : rupture_steps<double>(P, steps, D[p], T[p]);
-        if (rc) return rc;
     }
-    return FDPH_OK;
+    const int joined = batch_join(B);
+    return rc ? rc : joined;
 }
 
 int fdph_batch_synchronize(fdph_batch_t B) {
@@ -2552,7 +2577,13 @@ int fdph_batch_synchronize(fdph_batch_t B) {
 
 void fdph_batch_destroy(fdph_batch_t B) {
     if (!B) return;
-    for (fdph_plan_t P : B->plans) cudaStreamSynchronize(P->stream);
+    cudaSetDevice(B->device);
+    if (B->hub) {   // (behind the last call's work; the plans are not touched)
+        cudaStreamSynchronize(B->hub);
+        cudaStreamDestroy(B->hub);
+    }
+    if (B->ev_plan) cudaEventDestroy(B->ev_plan);
+    if (B->ev_hub) cudaEventDestroy(B->ev_hub);
     delete B;
 }
 
