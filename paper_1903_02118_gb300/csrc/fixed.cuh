@@ -206,10 +206,11 @@ __global__ void __launch_bounds__(32 * kFxWarps, B == 1 ? 5 : 3) fixed_block_ker
             double x[B];
             if (ai == 0) {
                 const double* Cr = a.Cring + rh * a.rs_C + col;
+                const bool fixed = a.hist != HIST_BASE || tk.W >= kBlk;   // (else rup_step_kernel takes the static term)
 #pragma unroll
                 for (int b = 0; b < B; ++b) {
                     const int tt = min(t0 + b, hist_end(a, n) - 1);   // (the slip by the steps that the launch may use)
-                    x[b] = b < nb && src && tt >= 0 ? Cr[(size_t)wrap(tt, a.WC) * a.N] : 0.0;
+                    x[b] = b < nb && src && fixed && tt >= 0 ? Cr[(size_t)wrap(tt, a.WC) * a.N] : 0.0;
                 }
             } else {
                 double* vs = a.vstate + rh * a.len_vstate + tk.vstate + (size_t)(ai - 1) * ns + (src ? lane : 0);

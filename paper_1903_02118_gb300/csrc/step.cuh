@@ -866,6 +866,7 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
         double* dw = (double*)mem;                                     // [B][32] slip rates D(n + b - W)
         R* vr = (R*)(dw + B * 32) + (size_t)grp * B * (span + 4);      // [B][span + 4] rows of the group's slice
         const int t0 = n - tk.W;
+        const bool fixed = a.hist != HIST_BASE || tk.W >= kBlk;   // (else rup_step_kernel takes the static term)
         const double* Dr = a.Dring + rh * a.rs_D + col;
         const double* Cr = a.Cring + rh * a.rs_C + col;
         double* vs = a.vstate + rh * a.len_vstate + tk.vstate + (src ? ri : 0);
@@ -886,7 +887,7 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
 #pragma unroll
                 for (int b = 0; b < B; ++b) {
                     const int t = min(t0 + b, hend - 1);   // (the slip by the steps that the launch may use)
-                    vr[b * (span + 4) + ri] = narrow(b < nb && src && t >= 0 ? Cr[(size_t)wrap(t, a.WC) * a.N] : 0.0, R());
+                    vr[b * (span + 4) + ri] = narrow(b < nb && src && fixed && t >= 0 ? Cr[(size_t)wrap(t, a.WC) * a.N] : 0.0, R());
                 }
             } else if (on) {
                 const double rho = a.rho[ai - 1];
@@ -959,9 +960,10 @@ struct FrictionDev {
 // slip rates before the step's aligned block [n0, n0 + kBlk) do, computed for the whole block
 // beforehand) plus what the block's own earlier steps n0 ... n - 1 do: by causality only the kernel
 // steps 1 ... n - n0 of the near leaves that a wave crosses that fast (RecLeaf: the first kz kernel
-// steps of a leaf vanish), and the static term of leaves with a window shorter than a block, on the slip
-// C(n - W) - C(n0 - 1) (the far blocks and the other static and tail terms act later than kBlk steps, see
-// rup_block).  One CTA per receiver group (the disjoint maximal receiver clusters of those leaves): its
+// steps of a leaf vanish), and the static term of leaves with a window shorter than a block, whole, on the
+// slip C(n - W) (the far blocks and the other static and tail terms act later than kBlk steps, see
+// rup_block; a share of it on the slip before the block would need C(n0 - 1), which neither the ring nor a
+// saved state holds where all windows are short).  One CTA per receiver group (the disjoint maximal receiver clusters of those leaves): its
 // warps take the (leaf, kernel step) units in turn, then the first warp solves the friction law and
 // appends the slip rate (push).  b: the step within the launch sequence's block.
 //
@@ -1007,7 +1009,7 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
     auto range = [&](const RecLeaf& L, int& first, int& steps) {
         first = max(L.kz, 1);
         steps = max(min(back + 1, L.W) - first, 0);
-        return steps + (L.stat >= 0 && back >= max(L.W, 1) ? 1 : 0);
+        return steps + (L.stat >= 0 && recent ? 1 : 0);
     };
     // the unit with running number r from leaf q on: its leaf (nleaf: none) and kernel step
     auto seek = [&](int& q, int r, int& k) {
@@ -1034,10 +1036,9 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
     auto load_v = [&](const RecLeaf& L, int k) -> R {
         const int c = L.s0 + min(lane, L.ns - 1);
         R v;
-        if (k < 0) {   // the slip of the block's steps up to n - W
-            const int t = min(n - L.W, n - 1), t0 = n - back - 1;
-            const double before = t0 >= 0 ? a.Cring[(size_t)wrap(t0, a.WC) * a.N + c] : 0.0;
-            v = narrow(a.Cring[(size_t)wrap(t, a.WC) * a.N + c] - before, R());
+        if (k < 0) {   // the slip of the steps up to n - W
+            const int t = min(n - L.W, n - 1);
+            v = narrow(t >= 0 ? a.Cring[(size_t)wrap(t, a.WC) * a.N + c] : 0.0, R());
         } else {
             const size_t off = (size_t)wrap(n - k, a.WD) * a.N + c;
             if constexpr (sizeof(R) == 4) v = a.Dring32[off]; else v = a.Dring[off];

@@ -71,3 +71,69 @@ def test_the_friction_law_is_the_one_last_given(batch):
         group.close()
     for p in plans:
         p.close()
+
+
+# Domain-S thresholds at which no window is longer than a few steps (0.5: none is kept at all)
+@pytest.mark.parametrize("prec", [fdph.FP64, fdph.FP32, fdph.FP16])
+@pytest.mark.parametrize("eps_st", [0.02, 0.05, 0.5])
+def test_short_windows(eps_st, prec):
+    """Rupture blocks of an operator whose windows are shorter than a block: the same bits step by step, and
+    from a state saved in the middle of a block; FP64 against predict / commit with the same law."""
+    _need_gpu()
+    N, M = 150, 90
+    law = (1.0, 0.6, 0.3, 2.0, 0)
+    tau0 = _tau0(N)
+
+    def plan():
+        p = _plan(N, prec, eps_st=eps_st)
+        assert p.stats()["max_window"] < 16
+        assert eps_st < 0.5 or p.stats()["max_window"] == 0
+        p.rupture_init(tau0, *law)
+        return p
+
+    def march(p, cuts, first=0):
+        D = torch.zeros((M, N), dtype=torch.float64, device="cuda")
+        T = torch.zeros_like(D)
+        torch.cuda.synchronize()
+        n = first
+        for m in cuts:
+            p.rupture_run(m, D[n:], T[n:])
+            n += m
+        p.synchronize()
+        return D.cpu().numpy(), T.cpu().numpy()
+
+    p = plan()
+    D, T = march(p, [M])
+    assert (D > 0).mean() > 0.05 and np.isfinite(T).all()
+    q = plan()
+    D1, T1 = march(q, [1] * M)
+    assert np.array_equal(D, D1) and np.array_equal(T, T1)
+    q.close()
+    for at in (21, 47):
+        q = plan()
+        march(q, [at])
+        state = q.save_state()
+        q.close()
+        q = plan()
+        q.load_state(state)
+        D2, T2 = march(q, [M - at], at)
+        assert np.array_equal(D[at:], D2[at:]) and np.array_equal(T[at:], T2[at:]), at
+        q.close()
+    if prec == fdph.FP64:
+        q = plan()
+        k0 = q.self_coefficients()
+        X = torch.zeros(N, dtype=torch.float64, device="cuda")
+        slip = np.zeros(N)
+        sigma_n, mu_s, mu_d, Dc, _ = law
+        for n in range(M):
+            q.predict(X)
+            q.synchronize()
+            tau = tau0.cpu().numpy() + X.cpu().numpy()
+            strength = sigma_n * (mu_s - (mu_s - mu_d) * np.minimum(slip / Dc, 1.0))
+            d = np.where(tau > strength, (tau - strength) / -k0, 0.0)
+            assert np.abs(d - D[n]).max() < 1e-9, n
+            q.commit(torch.from_numpy(d).cuda())
+            q.synchronize()
+            slip += d * 0.5
+        q.close()
+    p.close()
