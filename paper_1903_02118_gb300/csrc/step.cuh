@@ -729,10 +729,11 @@ struct NearCfg {
     using R = typename NearTypes<H>::Row;
     static constexpr int G = 4;                                       // window slices taken together
     static constexpr int pitch = 36;                                  // row of 32 entries, padded
-    // shared memory of one warp: the rows of a window item of `chunk` slices, or an aux item's
-    // slip rates (FP64) and one row of B steps for each of its lane groups' slices
+    // shared memory of one warp: the rows of a window item of `chunk` slices and, past 16 slices, its sums so
+    // far (FP64), or an aux item's slip rates (FP64) and one row of B steps for each of its lane groups' slices
     static constexpr size_t warp_bytes(int chunk) {
-        const size_t win = (size_t)((chunk + G - 1) / G * G + B - 1) * pitch * sizeof(R);
+        const size_t rows = (size_t)((chunk + G - 1) / G * G + B - 1) * pitch * sizeof(R);
+        const size_t win = (rows + 15) / 16 * 16 + (chunk > 16 ? (size_t)B * 32 * 8 : 0);
         const size_t aux = (size_t)B * 32 * 8 + (size_t)B * 64 * sizeof(R);
         return ((win > aux ? win : aux) + 15) / 16 * 16;
     }
@@ -743,8 +744,11 @@ struct NearCfg {
 // coefficients, the products bound the kernel, so what counts is how often the slip-rate rows are
 // read: window slice k of step n + b takes the row of step n + b - k, so the G slices of a group
 // meet only B + G - 1 rows, each read once (a broadcast) for up to G products.
-// Sums: 4 V-source groups of G slices in the row type, those over the slices of a group, then over the
-// groups; across items in FP64.
+// Sums in the row type: V sources of a slice, those of two slices over all sources, the two pairs of a group, up
+// to four groups; then FP64.  (A uniform slip rate cancels over the sources of a slice, not over the lags of a
+// source.  With V sources x 4 slices of a load in one sum the FP32 march of N = 300 without approximation was
+// 3.0e-7 off; this way it is 2.1e-7, and curved N = 4096 takes 2.23 instead of 2.17 ms per 64 steps.  One sum a
+// slice: 1.9e-7, but 64 sums in registers, 2.43 ms.)
 // Leaves of at most 16 receivers split the warp into 32 / span lane groups that take slices (window)
 // or aux slices of their own.
 template <class T, class H, int B>
@@ -809,46 +813,57 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
             R acc[B];
 #pragma unroll
             for (int b = 0; b < B; ++b) acc[b] = 0;
+            double* mid = (double*)(mem + warp_bytes) - B * 32;   // the sums so far, past 16 slices
+            const R ks = (R)a.kinv;   // the storage scale of the window (FP16), a power of two
             const int iters = (ngr + ngrp - 1) / ngrp;
             for (int i = 0; i < iters; ++i) {
                 const int gr = i * ngrp + grp;
                 const R* rg = rows + (size_t)min(gr, ngr - 1) * G * P;
-                R ga[B];
+                R s[2][B];   // sums of two slices each over the sources (see above)
 #pragma unroll
-                for (int b = 0; b < B; ++b) ga[b] = 0;
+                for (int b = 0; b < B; ++b) s[0][b] = s[1][b] = 0;
                 for (int jb = 0; jb < nbk; ++jb) {
                     R x[G][V];
 #pragma unroll
                     for (int g = 0; g < G; ++g) unpack(xn[g], x[g], R());
                     const bool wrapj = jb + 1 == nbk;
                     load(wrapj ? gr + ngrp : gr, wrapj ? 0 : jb + 1, xn);
-                    {
-                        R s[B];
 #pragma unroll
-                        for (int b = 0; b < B; ++b) s[b] = 0;
+                    for (int q = 0; q < B + G - 1; ++q) {
+                        R y[V];
+                        load_row<V>(rg + q * P + jb * V, y);
 #pragma unroll
-                        for (int q = 0; q < B + G - 1; ++q) {
-                            R y[V];
-                            load_row<V>(rg + q * P + jb * V, y);
+                        for (int g = 0; g < G; ++g) {
+                            const int b = B - 1 - q + g;
+                            if (b >= 0 && b < B) {
+                                constexpr int U = V < 4 ? V : 4;
+                                R t = x[g][0] * y[0];
 #pragma unroll
-                            for (int g = 0; g < G; ++g) {
-                                const int b = B - 1 - q + g;
-                                if (b >= 0 && b < B) {
+                                for (int v = 1; v < U; ++v) t = fma(x[g][v], y[v], t);
+                                if constexpr (V == 8) {
+                                    R u = x[g][4] * y[4];
 #pragma unroll
-                                    for (int v = 0; v < V; ++v) s[b] = fma(x[g][v], y[v], s[b]);
+                                    for (int v = 5; v < V; ++v) u = fma(x[g][v], y[v], u);
+                                    t += u;
                                 }
+                                s[g / 2][b] += t;
                             }
                         }
-#pragma unroll
-                        for (int b = 0; b < B; ++b) ga[b] += s[b];
                     }
                 }
 #pragma unroll
-                for (int b = 0; b < B; ++b) acc[b] += ga[b];
-            }
-            // window sums carry the storage scale of the window (FP16)
+                for (int b = 0; b < B; ++b) acc[b] += s[0][b] + s[1][b];
+                if ((i & 3) == 3 && i + 1 < iters) {
 #pragma unroll
-            for (int b = 0; b < B; ++b) tot[b] = wide(acc[b] * (R)a.kinv);   // (a power of two)
+                    for (int b = 0; b < B; ++b) {
+                        const double v = wide(acc[b] * ks);
+                        mid[b * 32 + lane] = i > 3 ? mid[b * 32 + lane] + v : v;
+                        acc[b] = 0;
+                    }
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < B; ++b) tot[b] = wide(acc[b] * ks) + (iters > 4 ? mid[b * 32 + lane] : 0.0);
         }
     } else {
         // aux slices: slice 0 the static tile (times C_j(n - W), it carries dt), slice 1 + q the tail

@@ -61,6 +61,8 @@ __device__ __forceinline__ void mma_16816_first(float (&c)[4], unsigned a0, unsi
 // 16 steps (near field 67 us a step); four, N = 2500, 1.69 -> 1.35 ms per 32.  One right-hand side was FP32 multiply-adds on the CUDA cores
 // (near_block_kernel): planar N = 1601, 502 -> 461 us per 32 steps.  Bound by latency and issue slots, not by
 // the tensor pipe: a slice is two 16-byte loads, then two (four) dependent MMAs and four FMAs a tile.
+static const int kSum = 8;   // slices of one FP32 sum; those go into a sum over the item
+
 template <int NR, int B>
 struct TcCfg {
     static constexpr int C = NR == 1 ? 4 : 2 * NR;            // columns of one row q
@@ -155,31 +157,45 @@ __global__ void __launch_bounds__(32 * TcCfg<NR, B>::warps, B == 1 ? 8 : 4) tc_b
     constexpr int parts = NR == 8 ? 2 : 1;   // (8 right-hand sides: the hi tile, then the lo tile)
     const __half* rk = rows + ((size_t)i0 * parts * 8 + g) * 32 + 8 * t;
     const float* sk = scl + i0 * parts * 8 + 2 * t;
-    for (int k = 0; k < nk; ++k, rk += C * 32, sk += C) {
-        const uint4 x0 = xn[0][0], x1 = xn[0][1];
+    float sum[T][4];   // of the parts before this one
 #pragma unroll
-        for (int d = 0; d + 1 < D; ++d) {
-            xn[d][0] = xn[d + 1][0];
-            xn[d][1] = xn[d + 1][1];
-        }
-        load(k + D, xn[D - 1]);
+    for (int i = 0; i < T; ++i)
 #pragma unroll
-        for (int i = 0; i < T; ++i) {
-            if (i >= nt) break;   // (warp-uniform)
-            float c[4];
+        for (int f = 0; f < 4; ++f) sum[i][f] = 0.f;
+    for (int k0 = 0; k0 < nk; k0 += kSum) {
+        for (int k = k0; k < min(k0 + kSum, nk); ++k, rk += C * 32, sk += C) {
+            const uint4 x0 = xn[0][0], x1 = xn[0][1];
 #pragma unroll
-            for (int h = 0; h < parts; ++h) {
-                const uint4 b = *(const uint4*)(rk + (size_t)(i * parts + h) * 8 * 32);
-                if (h == 0) mma_16816_first(c, x0.x, x1.x, x0.y, x1.y, b.x, b.y);
-                else mma_16816(c, x0.x, x1.x, x0.y, x1.y, b.x, b.y);
-                mma_16816(c, x0.z, x1.z, x0.w, x1.w, b.z, b.w);
+            for (int d = 0; d + 1 < D; ++d) {
+                xn[d][0] = xn[d + 1][0];
+                xn[d][1] = xn[d + 1][1];
             }
-            const float2 s = *(const float2*)(sk + i * parts * 8);
-            acc[i][0] = fmaf(c[0], s.x, acc[i][0]);
-            acc[i][1] = fmaf(c[1], s.y, acc[i][1]);
-            acc[i][2] = fmaf(c[2], s.x, acc[i][2]);
-            acc[i][3] = fmaf(c[3], s.y, acc[i][3]);
+            load(k + D, xn[D - 1]);
+#pragma unroll
+            for (int i = 0; i < T; ++i) {
+                if (i >= nt) break;   // (warp-uniform)
+                float c[4];
+#pragma unroll
+                for (int h = 0; h < parts; ++h) {
+                    const uint4 b = *(const uint4*)(rk + (size_t)(i * parts + h) * 8 * 32);
+                    if (h == 0) mma_16816_first(c, x0.x, x1.x, x0.y, x1.y, b.x, b.y);
+                    else mma_16816(c, x0.x, x1.x, x0.y, x1.y, b.x, b.y);
+                    mma_16816(c, x0.z, x1.z, x0.w, x1.w, b.z, b.w);
+                }
+                const float2 s = *(const float2*)(sk + i * parts * 8);
+                acc[i][0] = fmaf(c[0], s.x, acc[i][0]);
+                acc[i][1] = fmaf(c[1], s.y, acc[i][1]);
+                acc[i][2] = fmaf(c[2], s.x, acc[i][2]);
+                acc[i][3] = fmaf(c[3], s.y, acc[i][3]);
+            }
         }
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {
+                sum[i][f] += acc[i][f];
+                acc[i][f] = 0.f;
+            }
     }
     const bool fits = FDPH_IDX((long long)tk.item * 32 + 32 <= a.cap_partial, a.err);
     const float ks = a.kinv;   // the window's storage scale (a power of two)
@@ -189,9 +205,9 @@ __global__ void __launch_bounds__(32 * TcCfg<NR, B>::warps, B == 1 ? 8 : 4) tc_b
         if (i >= nt) break;
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
-            float v = acc[i][f];
+            float v = sum[i][f];
             if constexpr (NR == 4) v += __shfl_xor_sync(0xffffffffu, v, 2);   // hi + lo
-            if constexpr (NR == 1) v += acc[i][f ^ 1];                         // hi + lo, rest + 0
+            if constexpr (NR == 1) v += sum[i][f ^ 1];                         // hi + lo, rest + 0
             if constexpr (NR <= 2) v += __shfl_xor_sync(0xffffffffu, v, 1);
             const int col = 2 * t + (f & 1);          // column of the tile
             const int q = Cf::per * (i0 + i) + (NR <= 2 ? col >> 2 : 0), r = col % NR, b = S - 1 - q;
