@@ -4,8 +4,9 @@
 // scatter and transient + Eq. 39 on two side streams, beside the near field, all joined before the gather.
 // Causality (min(dm + delay) >= 1, checked at plan time) guarantees that the ring slots read at step n were
 // completed by steps < n and that the slots written at step n are not read; where min(dm + delay) is less
-// than the block's length, Eq. 39 follows the scatter.  The near field runs on the CUDA cores (FP32, step.cuh)
-// or on the tensor cores (FP16 windows, tensor.cuh; FP64 by exact products, fixed.cuh).  Several right-hand
+// than the block's length, Eq. 39 follows the scatter.  The near field runs on the CUDA cores (FP32, and
+// FP16 windows of one right-hand side, step.cuh) or on the tensor cores (FP16 windows of several, tensor.cuh; FP64,
+// fixed.cuh).  Several right-hand
 // sides go through one launch.  A rupture block (Sec. 6.2) takes what the slip rates before the block do to
 // all its steps at once, then step by step its own part, the friction law and the push, then commits the
 // block.  A batch runs its plans on their own streams.
@@ -560,7 +561,10 @@ static void launch_tc(const StepArgs<float>& a, int n_win, int chunk, cudaStream
     tc_block_kernel<NR, B><<<n_win, 32 * TcCfg<NR, B>::warps, TcCfg<NR, B>::smem(chunk), s>>>(a, chunk);
 }
 
-// The near field of a launch: the window items (FP16 plans), or all items (FP64 and FP32 plans)
+// The near field of a launch: the window items (FP16 plans), or all items (FP64 and FP32 plans).  FP16 windows of
+// one right-hand side meet FP32 slip rates on the CUDA cores: on the tensor cores, as three FP16 parts under a
+// common scale, slip rates below 2^-15 of the leaf's largest lost digits (planar N = 1601, 32 steps: 461 us
+// there, 545 us here).
 template <class T>
 static void launch_near(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
     if (!a.n_items) return;
@@ -571,11 +575,13 @@ static void launch_near(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
     } else if (P->precision == FDPH_FP16) {
         if (!P->n_win) return;
         const bool one = a.nb == 1;
+        StepArgs<T> w = a;   // (one right-hand side)
+        w.n_items = P->n_win;
         switch (P->nrhs) {
             case 2: one ? launch_tc<2, 1>(a, P->n_win, P->chunk, s) : launch_tc<2, kBlk>(a, P->n_win, P->chunk, s); break;
             case 4: one ? launch_tc<4, 1>(a, P->n_win, P->chunk, s) : launch_tc<4, kBlk>(a, P->n_win, P->chunk, s); break;
             case 8: one ? launch_tc<8, 1>(a, P->n_win, P->chunk, s) : launch_tc<8, kBlk>(a, P->n_win, P->chunk, s); break;
-            default: one ? launch_tc<1, 1>(a, P->n_win, P->chunk, s) : launch_tc<1, kBlk>(a, P->n_win, P->chunk, s);
+            default: one ? launch_near_items<T, __half, 1>(w, P->chunk, s) : launch_near_items<T, __half, kBlk>(w, P->chunk, s);
         }
     } else if (a.nb == 1) {
         launch_near_items<T, float, 1>(a, P->chunk, s);
@@ -988,9 +994,11 @@ static int build_schedule(fdph_plan_t P) {
     std::vector<NearTask> tasks(ni);
     for (int q = 0; q < ni; ++q) tasks[q] = all[order[q]];
     // shared memory of the near kernels for items of this length
-    if (tc) {
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<1, 1>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<1, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<1, kBlk>::smem(kChunk)));
+    if constexpr (std::is_same<H, __half>::value) {
+        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, H, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)NearCfg<H, 1>::warp_bytes(kChunk) * kNearWarps));
+        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, H, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)NearCfg<H, kBlk>::warp_bytes(kChunk) * kNearWarps));
         FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<2, 1>::smem(kChunk)));
         FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<2, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<2, kBlk>::smem(kChunk)));
         FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<4, 1>::smem(kChunk)));
@@ -1126,8 +1134,8 @@ static int build_near_begin(fdph_plan_t P, const PlanInputs& in, NearBuild& nb) 
         kz[l] = std::min(kz[l], W[l]);
         slices += std::max(W[l] - kz[l], 1);
     }
-    // (an item is a CTA's work on the tensor cores: FP64 and FP16 plans)
-    const bool cta = P->precision != FDPH_FP32;
+    // (an item is a CTA's work on the tensor cores: FP64, and FP16 with several right-hand sides)
+    const bool cta = P->precision == FDPH_FP64 || (P->precision == FDPH_FP16 && P->nrhs > 1);
     int chunk = std::min(near_max_chunk(P->nrhs, P->precision), kChunk / 2);
     while (chunk > 8 / std::min(P->nrhs, 2) && slices * P->nrhs / chunk < 4LL * 152 * (cta ? 3 : 16)) chunk /= 2;
     P->aux_chunk = near_aux_chunk(P->precision, nl);

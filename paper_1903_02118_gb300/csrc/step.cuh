@@ -674,7 +674,8 @@ __global__ void gather_kernel(StepArgs<T> a0) {
     }
 }
 
-// ---- near field (App. E) on the CUDA cores (FP32 items; FP16 windows: tensor.cuh, FP64 plans: fixed.cuh)
+// ---- near field (App. E) on the CUDA cores: FP32 items, FP16 windows of one right-hand side (several:
+// tensor.cuh; FP64 plans: fixed.cuh)
 
 // Near-field storage: window slices in H; aux slices (static tile, tail coefficients) in the aux
 // type (FP32 when the window is FP16: the static term multiplies the cumulative slip, so its
@@ -825,7 +826,10 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
                 for (int jb = 0; jb < nbk; ++jb) {
                     R x[G][V];
 #pragma unroll
-                    for (int g = 0; g < G; ++g) unpack(xn[g], x[g], R());
+                    for (int g = 0; g < G; ++g) {
+                        if constexpr (sizeof(H) == 2) unpack(xn[g], x[g], __half());
+                        else unpack(xn[g], x[g], R());
+                    }
                     const bool wrapj = jb + 1 == nbk;
                     load(wrapj ? gr + ngrp : gr, wrapj ? 0 : jb + 1, xn);
 #pragma unroll
@@ -865,7 +869,7 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
 #pragma unroll
             for (int b = 0; b < B; ++b) tot[b] = wide(acc[b] * ks) + (iters > 4 ? mid[b * 32 + lane] : 0.0);
         }
-    } else {
+    } else if constexpr (sizeof(H) != 2) {   // (those of FP16 plans go to the FP32 instance)
         // aux slices: slice 0 the static tile (times C_j(n - W), it carries dt), slice 1 + q the tail
         // coefficients of term q (times the tail state V_qj(n) = rho_q V_qj(n - 1) + D_{j, n-W}, updated
         // here by its only reader).  Lane j of a lane group forms its slice's rows of the B steps.

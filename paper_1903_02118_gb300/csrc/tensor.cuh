@@ -1,4 +1,4 @@
-// tensor.cuh -- the near-field windows of FP16 plans on the tensor cores.
+// tensor.cuh -- the near-field windows of FP16 plans with several right-hand sides on the tensor cores.
 //
 // One window slice is a 32 x 32 (receivers x sources) FP16 tile; with the R right-hand sides and the B
 // steps of a launch it meets R B slip-rate rows: a dense (32 x 32) x (32 x R B) contraction, run as
@@ -11,14 +11,13 @@
 // lane t, the A fragments of lane (g, t) are exactly the stored 16 bytes (sources 8 t ... 8 t + 7 of one
 // receiver, plan.h), and the B fragments of both 16-source steps are 16 contiguous bytes of a row.
 //
-// The slip rates must not lose digits to FP16: the 32 sources of a row (step, right-hand side) are split into
-// two FP16 rows of x 2^sh (sh puts the largest of them in [2^13, 2^14); hi = fp16(x 2^sh), lo =
-// fp16(x 2^sh - hi), 2^-22 relative, 2^-39 of the largest absolute), separate columns of the contraction, so
-// that the only rounding of the FP16 path remains that of the stored coefficients.  One right-hand side has
-// columns to spare and carries a third part, fp16 of what hi and lo leave: the FP32 slip rate.  Each slice's
-// products are scaled back per column by 2^-sh and added to the item's FP32 sums.  (The scale is of the
-// leaf's own sources, found by the warp that stages them: one scale for a whole step's slip rates took a
-// kernel between the push and the near field and lost digits where a leaf is quiet.)
+// The slip rates go in with more digits than FP16 has: the 32 sources of a row (step, right-hand side) are split
+// into two FP16 rows of x 2^sh (sh puts the largest of them in [2^13, 2^14); hi = fp16(x 2^sh), lo =
+// fp16(x 2^sh - hi)), separate columns of the contraction.  A slip rate keeps 2^-22 of itself, but no less than 2^-39
+// of the largest of the leaf's 32 sources: one at 1e-6 of it is good to 2e-6.  Each slice's products are scaled
+// back per column by 2^-sh and added to the item's FP32 sums.  (The scale is of the leaf's own sources, found by
+// the warp that stages them: one scale for a whole step's slip rates took a kernel between the push and the
+// near field and lost digits where a leaf is quiet.)
 #pragma once
 #include "step.cuh"
 
@@ -50,23 +49,26 @@ __device__ __forceinline__ void mma_16816_first(float (&c)[4], unsigned a0, unsi
 
 // NR right-hand sides, B steps of a launch (1 or 16).  Rows in shared memory: row q of the item holds the slip
 // rates of step n + S - 1 - k0 - q, S the steps rounded up to whole tiles, [q][part][right-hand side][32 sources] with
-// the parts hi, lo (one right-hand side: hi, lo, rest, zero); 8 consecutive rows are the columns of one MMA
-// tile, so window slice k takes the tiles from row k - k0 on (tile = one step of 8 right-hand sides' hi or
-// lo, of 4 with both, 2 steps of 2 or of one with its four parts).
+// the parts hi, lo; 8 consecutive rows are the columns of one MMA tile, so window slice k takes the tiles from
+// row k - k0 on (tile = one step of 8 right-hand sides' hi or lo, of 4 with both, 2 steps of 2).
 //
 // Warps take 16 receivers and a share of the tiles each, and all slices of the item: the item's sums stay in
 // the accumulators and are written straight out, and 16 steps of 8 right-hand sides take one pass over the
 // coefficients.  With a share of the slices per warp the sums of the four warps met in shared memory and FP64
 // at the end of every item, and two passes were needed: eight right-hand sides, N = 6000, 3.86 -> 3.23 ms per
-// 16 steps (near field 67 us a step); four, N = 2500, 1.69 -> 1.35 ms per 32.  One right-hand side was FP32 multiply-adds on the CUDA cores
-// (near_block_kernel): planar N = 1601, 502 -> 461 us per 32 steps.  Bound by latency and issue slots, not by
-// the tensor pipe: a slice is two 16-byte loads, then two (four) dependent MMAs and four FMAs a tile.
-static const int kSum = 8;   // slices of one FP32 sum; those go into a sum over the item
+// 16 steps (near field 67 us a step); four, N = 2500, 1.69 -> 1.35 ms per 32.  Bound by latency and issue slots,
+// not by the tensor pipe: a slice is two 16-byte loads, then two (four) dependent MMAs and four FMAs a tile.
+//
+// The FP32 sum of a slice's products goes into a sum over kSum slices, that into a sum over the item.  (Against exact
+// sums of the stored coefficients, plain march of N = 300, noise, four right-hand sides: one sum over the item
+// 1.35e-7, kSum = 16, 8, 4: 1.18, 1.10, 1.10e-7.  Parts that meet in FP64 in the item's partial sum take four right-hand
+// sides of N = 2500 from 1.36 to 1.53 ms.)
+static const int kSum = 8;
 
 template <int NR, int B>
 struct TcCfg {
-    static constexpr int C = NR == 1 ? 4 : 2 * NR;            // columns of one row q
-    static constexpr int per = NR <= 2 ? 8 / C : 1;           // steps of one tile
+    static constexpr int C = 2 * NR;                          // columns of one row q
+    static constexpr int per = NR == 2 ? 2 : 1;               // steps of one tile
     static constexpr int S = B < per ? per : B;
     static constexpr int tiles = S / per;                     // accumulator tiles (hi and lo of 8 share one)
     static constexpr int warps = B == 1 ? 2 : 4;
@@ -118,10 +120,6 @@ __global__ void __launch_bounds__(32 * TcCfg<NR, B>::warps, B == 1 ? 8 : 4) tc_b
                     __half* row = rows + (size_t)((q0 + i) * C + r) * 32 + lane;
                     row[0] = hi;
                     row[NR * 32] = lo;
-                    if constexpr (NR == 1) {
-                        row[64] = __float2half_rn(y1 - __half2float(lo));
-                        row[96] = __float2half_rn(0.f);
-                    }
                     if (lane < C / NR) scl[(q0 + i) * C + lane * NR + r] = pow2f(-sh);
                 }
             }
@@ -207,11 +205,10 @@ __global__ void __launch_bounds__(32 * TcCfg<NR, B>::warps, B == 1 ? 8 : 4) tc_b
         for (int f = 0; f < 4; ++f) {
             float v = sum[i][f];
             if constexpr (NR == 4) v += __shfl_xor_sync(0xffffffffu, v, 2);   // hi + lo
-            if constexpr (NR == 1) v += sum[i][f ^ 1];                         // hi + lo, rest + 0
-            if constexpr (NR <= 2) v += __shfl_xor_sync(0xffffffffu, v, 1);
+            if constexpr (NR == 2) v += __shfl_xor_sync(0xffffffffu, v, 1);
             const int col = 2 * t + (f & 1);          // column of the tile
-            const int q = Cf::per * (i0 + i) + (NR <= 2 ? col >> 2 : 0), r = col % NR, b = S - 1 - q;
-            const bool mine = NR == 8 || (NR == 4 ? col < 4 : NR == 2 ? !(col & 2) : !(col & 3));
+            const int q = Cf::per * (i0 + i) + (NR == 2 ? col >> 2 : 0), r = col % NR, b = S - 1 - q;
+            const bool mine = NR == 8 || (NR == 4 ? col < 4 : !(col & 2));
             const int row = g + 8 * (f >> 1);
             if (mine && fits && b < nb && 16 * mt + row < nr) out[r * a.rs_partial + b * a.cap_partial + row] = wide(v * ks);
         }
