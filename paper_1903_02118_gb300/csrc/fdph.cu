@@ -4,9 +4,8 @@
 // scatter and transient + Eq. 39 on two side streams, beside the near field, all joined before the gather.
 // Causality (min(dm + delay) >= 1, checked at plan time) guarantees that the ring slots read at step n were
 // completed by steps < n and that the slots written at step n are not read; where min(dm + delay) is less
-// than the block's length, Eq. 39 follows the scatter.  The near field runs on the CUDA cores (FP32, and
-// FP16 windows of one right-hand side, step.cuh) or on the tensor cores (FP16 windows of several, tensor.cuh; FP64,
-// fixed.cuh).  Several right-hand
+// than the block's length, Eq. 39 follows the scatter.  The near field runs on the CUDA cores (FP64, FP32, and
+// FP16 windows of one right-hand side, step.cuh) or on the tensor cores (FP16 windows of several, tensor.cuh).  Several right-hand
 // sides go through one launch.  A rupture block (Sec. 6.2) takes what the slip rates before the block do to
 // all its steps at once, then step by step its own part, the friction law and the push, then commits the
 // block.  A batch runs its plans on their own streams.
@@ -30,7 +29,6 @@
 #include "../../include/fdph.h"
 #include "internal.h"
 #include "kernel2d.cuh"
-#include "fixed.cuh"
 #include "plan.h"
 #include "step.cuh"
 #include "tensor.cuh"
@@ -98,13 +96,11 @@ static inline int near_max_chunk(int nrhs, int precision) {
     return (nrhs >= 2 && precision != FDPH_FP64 ? 2 * kChunk : kChunk) / nrhs;
 }
 
-// the longest aux item: all of a leaf's static tile and tail slices, or half of them where one warp takes an
-// item and there is less than one leaf per scheduler (152 SMs x 4): one item of all 17 slices then takes as
+// the longest aux item: all of a leaf's static tile and tail slices, or half of them where
+// there is less than one leaf per scheduler (152 SMs x 4): one item of all 17 slices then takes as
 // long as the rest of the step (curved N = 1024, 422 leaves: 0.95 -> 0.80 ms per 64 steps; with 1963 leaves the
 // split costs 2.18 -> 2.38 ms)
-static inline int near_aux_chunk(int precision, int leaves) {
-    return precision == FDPH_FP64 || leaves >= 4 * 152 ? 1 + kMaxSoe : 9;
-}
+static inline int near_aux_chunk(int leaves) { return leaves >= 4 * 152 ? 1 + kMaxSoe : 9; }
 
 // ------------------------------------------------------------------------------------------
 // plan-time device kernels: near-field windows and exact-kernel tensors
@@ -287,9 +283,6 @@ struct fdph_plan_s {
     int n_win = 0, n_aux = 0; // window and aux items (tensor cores: the window items first)
     void* tensor = nullptr;
     void* stat = nullptr;     // aux slices, storage type
-    int *fx_win = nullptr, *fx_aux = nullptr;   // FP64: slice exponents (fixed.cuh)
-    double* rec_tensor = nullptr;               // FP64: the rupture leaves' first kBlk kernel steps as numbers
-    long long rec_len = 0;
     int *np_ptr = nullptr, *np_idx = nullptr;
     int* err = nullptr;
     double* rho = nullptr;
@@ -461,10 +454,6 @@ static StepArgs<T> make_args(fdph_plan_t P, const double* D, double* T_) {
     a.n_items = P->n_win + P->n_aux;
     a.tensor = P->tensor;
     a.kinv = (float)(1.0 / P->kscale);
-    a.fx_win = P->fx_win;
-    a.fx_aux = P->fx_aux;
-    a.rec_tensor = P->rec_tensor ? P->rec_tensor : P->tensor;
-    a.len_rec = P->rec_tensor ? P->rec_len : hp.near_tensor_len;
     a.stat = P->stat;
     a.len_tensor = hp.near_tensor_len;
     a.len_aux = hp.near_aux_len;
@@ -568,10 +557,9 @@ static void launch_tc(const StepArgs<float>& a, int n_win, int chunk, cudaStream
 template <class T>
 static void launch_near(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
     if (!a.n_items) return;
-    if constexpr (sizeof(T) == 8) {   // exact products on the tensor cores
-        const dim3 g(a.n_items, a.nrhs);
-        if (a.nb == 1) fixed_block_kernel<1><<<g, 32 * kFxWarps, FxCfg<1>::smem(P->chunk), s>>>(a, P->chunk);
-        else fixed_block_kernel<kBlk><<<g, 32 * kFxWarps, FxCfg<kBlk>::smem(P->chunk), s>>>(a, P->chunk);
+    if constexpr (sizeof(T) == 8) {
+        if (a.nb == 1) launch_near_items<T, double, 1>(a, P->chunk, s);
+        else launch_near_items<T, double, kBlk>(a, P->chunk, s);
     } else if (P->precision == FDPH_FP16) {
         if (!P->n_win) return;
         const bool one = a.nb == 1;
@@ -940,16 +928,6 @@ static int launch_commit(fdph_plan_t P, const double* D_n) {
     return FDPH_OK;
 }
 
-// first slice of every leaf among the plan's window and aux slices
-static void slice_numbers(const HostPlan& hp, std::vector<long long>& win0, std::vector<long long>& aux0) {
-    win0.assign(1, 0);
-    aux0.assign(1, 0);
-    for (const NearLeaf& L : hp.near) {
-        win0.push_back(win0.back() + L.W);
-        aux0.push_back(aux0.back() + L.naux);
-    }
-}
-
 // The plan's near-field work items as the near kernels read them: window items first where they go to
 // the tensor cores, else all together, largest first (an item is a warp's or a CTA's work: the last to
 // start are the shortest).
@@ -961,8 +939,6 @@ static int build_schedule(fdph_plan_t P) {
     const int ni = (int)hp.items.size();
     std::vector<NearTask> all(ni);
     std::vector<double> cost(ni);
-    std::vector<long long> win0, aux0;
-    slice_numbers(hp, win0, aux0);
     P->n_win = P->n_aux = 0;
     for (int q = 0; q < ni; ++q) {
         const NearItem& it = hp.items[q];
@@ -980,7 +956,6 @@ static int build_schedule(fdph_plan_t P) {
         t.s0 = L.s0;
         t.W = L.W;
         t.vstate = (int)L.vstate;
-        t.slice = it.k0 + (int)(it.kind ? aux0[it.leaf] : win0[it.leaf]);
         // bytes, and for aux slices the FP64 work of their rows and sums
         cost[q] = (double)(it.k1 - it.k0) * (t.sl * (double)(it.kind ? sizeof(A) : sizeof(H)) + (it.kind ? 4096.0 : 0.0)) + 4096.0;
         (it.kind ? P->n_aux : P->n_win) += 1;
@@ -1006,15 +981,12 @@ static int build_schedule(fdph_plan_t P) {
         FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8, 1>::smem(kChunk)));
         FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8, kBlk>::smem(kChunk)));
     }
-    if constexpr (sizeof(H) == 8) {
-        FDPH_CUDA(cudaFuncSetAttribute(fixed_block_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FxCfg<1>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(fixed_block_kernel<kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FxCfg<kBlk>::smem(kChunk)));
-    } else {
-        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, float, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)NearCfg<float, 1>::warp_bytes(2 * kChunk) * kNearWarps));
-        FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, float, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)NearCfg<float, kBlk>::warp_bytes(2 * kChunk) * kNearWarps));
-    }
+    constexpr int longest = sizeof(H) == 8 ? kChunk : 2 * kChunk;   // (near_max_chunk)
+    using I = typename std::conditional<sizeof(H) == 8, double, float>::type;
+    FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, I, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)NearCfg<I, 1>::warp_bytes(longest) * kNearWarps));
+    FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, I, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)NearCfg<I, kBlk>::warp_bytes(longest) * kNearWarps));
     P->sched_version += 1;
     int rc;
     if ((rc = upload(P, &P->tasks, tasks)) || (rc = upload(P, &P->np_ptr, hp.np_ptr)) || (rc = upload(P, &P->np_idx, hp.np_idx)))
@@ -1134,11 +1106,11 @@ static int build_near_begin(fdph_plan_t P, const PlanInputs& in, NearBuild& nb) 
         kz[l] = std::min(kz[l], W[l]);
         slices += std::max(W[l] - kz[l], 1);
     }
-    // (an item is a CTA's work on the tensor cores: FP64, and FP16 with several right-hand sides)
-    const bool cta = P->precision == FDPH_FP64 || (P->precision == FDPH_FP16 && P->nrhs > 1);
+    // (an item is a CTA's work on the tensor cores: FP16 with several right-hand sides)
+    const bool cta = P->precision == FDPH_FP16 && P->nrhs > 1;
     int chunk = std::min(near_max_chunk(P->nrhs, P->precision), kChunk / 2);
     while (chunk > 8 / std::min(P->nrhs, 2) && slices * P->nrhs / chunk < 4LL * 152 * (cta ? 3 : 16)) chunk /= 2;
-    P->aux_chunk = near_aux_chunk(P->precision, nl);
+    P->aux_chunk = near_aux_chunk(nl);
     finish_near_layout(hp, W, kz, has_tail, chunk, 16 / (int)sizeof(H), 16 / (int)sizeof(A), P->aux_chunk);
     P->near_W = W;
     P->near_kz = kz;
@@ -1215,10 +1187,8 @@ static int build_near_begin(fdph_plan_t P, const PlanInputs& in, NearBuild& nb) 
     return FDPH_OK;
 }
 
-// near leaves that act within a rupture block, and what rec_tensor keeps of one: its kernel steps below
-// kBlk, and the static tile of a shorter window
+// near leaves that act within a rupture block
 static bool rec_leaf(const NearLeaf& L) { return L.kz < kBlk || (L.W < kBlk && L.tail < 0); }
-static long long rec_size(const NearLeaf& L) { return L.W < kBlk ? (long long)L.W * L.sl + L.sla : (long long)kBlk * L.sl; }
 
 template <class T, class H>
 static int build_near_finish(fdph_plan_t P, const PlanInputs& in, NearBuild& nb) {
@@ -1263,35 +1233,6 @@ static int build_near_finish(fdph_plan_t P, const PlanInputs& in, NearBuild& nb)
                                       cudaMemcpyHostToDevice, P->stream));
     }
     stamp("near: tail fits");
-    if constexpr (sizeof(H) == 8) {
-        // the rupture leaves' first kernel steps stay as numbers; then all slices take the form of fixed.cuh
-        for (const NearLeaf& L : hp.near)
-            if (rec_leaf(L)) P->rec_len += rec_size(L);
-        if ((rc = dalloc(P, &P->rec_tensor, (size_t)P->rec_len))) return rc;
-        long long at = 0;
-        for (const NearLeaf& L : hp.near)
-            if (rec_leaf(L)) {
-                const size_t c = (size_t)std::min(L.W, kBlk) * L.sl;
-                if (c) FDPH_CUDA(cudaMemcpyAsync(P->rec_tensor + at, (const double*)P->tensor + L.tensor, c * sizeof(double),
-                                                 cudaMemcpyDeviceToDevice, P->stream));
-                if (L.W < kBlk)
-                    FDPH_CUDA(cudaMemcpyAsync(P->rec_tensor + at + c, (const double*)P->stat + L.stat, L.sla * sizeof(double),
-                                              cudaMemcpyDeviceToDevice, P->stream));
-                at += rec_size(L);
-            }
-        std::vector<long long> win0, aux0;
-        slice_numbers(hp, win0, aux0);
-        long long *d_win0 = nullptr, *d_aux0 = nullptr;
-        if ((rc = upload(P, &d_win0, win0)) || (rc = upload(P, &d_aux0, aux0)) || (rc = dalloc(P, &P->fx_win, (size_t)win0.back() * 2)) ||
-            (rc = dalloc(P, &P->fx_aux, (size_t)aux0.back() * 2)))
-            return rc;
-        const int nl = (int)hp.near.size();
-        if (nl) {
-            fx_pack_kernel<<<nl, 256, 0, P->stream>>>((double*)P->tensor, P->fx_win, P->near, d_win0, 0, hp.soe);
-            fx_pack_kernel<<<nl, 256, 0, P->stream>>>((double*)P->stat, P->fx_aux, P->near, d_aux0, 1, hp.soe);
-            FDPH_CUDA(cudaGetLastError());
-        }
-    }
     if ((rc = build_schedule<T, H>(P))) return rc;
     FDPH_CUDA(cudaStreamSynchronize(P->stream));
     return FDPH_OK;
@@ -1332,21 +1273,13 @@ static int build_recent(fdph_plan_t P) {
     std::vector<RecLeaf> leaves;
     std::vector<std::vector<int>> per(groups.size());
     for (int l : use) per[group_of[hp.near[l].r0]].push_back(l);
-    std::vector<long long> at(hp.near.size(), 0);   // FP64: place in rec_tensor
-    if (P->rec_tensor) {
-        long long o = 0;
-        for (int l : use) {
-            at[l] = o;
-            o += rec_size(hp.near[l]);
-        }
-    }
     for (size_t g = 0; g < groups.size(); ++g) {
         groups[g].leaf0 = (int)leaves.size();
         groups[g].nleaf = (int)per[g].size();
         for (int l : per[g]) {
             const NearLeaf& L = hp.near[l];
-            const long long stat = L.W < kBlk && L.tail < 0 ? (P->rec_tensor ? at[l] + (long long)L.W * L.sl : (long long)L.stat) : -1;
-            leaves.push_back({P->rec_tensor ? at[l] : (long long)L.tensor, stat, L.sl, L.r0, L.nr, L.s0, L.ns, L.kz, L.W, 0});
+            const long long stat = L.W < kBlk && L.tail < 0 ? (long long)L.stat : -1;
+            leaves.push_back({(long long)L.tensor, stat, L.sl, L.r0, L.nr, L.s0, L.ns, L.kz, L.W, 0});
         }
     }
     P->n_groups = (int)groups.size();
@@ -1427,7 +1360,7 @@ static void fill_stats(fdph_plan_t P) {
     s.state_bytes = (long long)P->state_bytes;
     long long arena = 0;
     arena += (long long)(hp.fac.size() * ps) + hp.ints.size() * 4 + hp.sbs.size() * sizeof(SbDev);
-    arena += (long long)(hp.near_tensor_len * pw + hp.near_aux_len * ps) + P->rec_len * 8;
+    arena += (long long)(hp.near_tensor_len * pw + hp.near_aux_len * ps);
     s.arena_bytes = arena;
 }
 

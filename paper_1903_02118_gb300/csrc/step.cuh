@@ -63,8 +63,7 @@ struct NearDev {
 struct __align__(16) NearTask {
     long long off;       // element offset of the item's first slice (tensor, or aux for kind 1)
     int item, k0, k1, kind, nr, ns, sl, s0, W, vstate;
-    int slice;           // FP64 plans: number of the item's first slice among the plan's slices of its kind
-    int pad;
+    int pad[2];
 };
 static_assert(sizeof(NearTask) == 64, "one work item is four 16-byte loads");
 
@@ -90,8 +89,8 @@ struct RecGroup {
     int r0, nr, leaf0, nleaf;
 };
 struct __align__(16) RecLeaf {
-    long long off;       // element offset of kernel step 0 in rec_tensor
-    long long stat;      // W < kBlk: the static tile, in rec_tensor (FP64) or the aux slices; else -1
+    long long off;       // element offset of kernel step 0 in the window slices
+    long long stat;      // W < kBlk: the static tile among the aux slices; else -1
     int sl, r0, nr, s0, ns, kz, W, pad;
 };
 static_assert(sizeof(RecLeaf) == 48, "a leaf is three 16-byte loads");
@@ -153,11 +152,8 @@ struct StepArgs {
     int n_items;
     const void* tensor;       // near-field window slices (window storage type)
     float kinv;               // inverse of the window coefficients' storage scale (FP16: 2^-e, else 1)
-    const int *fx_win, *fx_aux;   // FP64 plans: exponents of the slices (fixed.cuh), [slice][2]
-    const void* rec_tensor;   // the kernel steps of a rupture block's own part (RecLeaf::off), window storage
-                              // type (FP64 plans: as numbers, not in the form of fixed.cuh)
     const void* stat;         // aux slices: static tiles, exponential-tail coefficients (aux storage type)
-    long long len_tensor, len_aux, len_rec;   // elements of tensor, stat and rec_tensor (index checks of FDPH_CHECK builds)
+    long long len_tensor, len_aux;   // elements of tensor and stat (index checks of FDPH_CHECK builds)
     double* partial;          // [kBlk][cap_partial]: [item][32] per step
     long long cap_partial;
     const int* np_ptr;
@@ -674,8 +670,8 @@ __global__ void gather_kernel(StepArgs<T> a0) {
     }
 }
 
-// ---- near field (App. E) on the CUDA cores: FP32 items, FP16 windows of one right-hand side (several:
-// tensor.cuh; FP64 plans: fixed.cuh)
+// ---- near field (App. E) on the CUDA cores: FP64 and FP32 items, FP16 windows of one right-hand side (several:
+// tensor.cuh)
 
 // Near-field storage: window slices in H; aux slices (static tile, tail coefficients) in the aux
 // type (FP32 when the window is FP16: the static term multiplies the cumulative slip, so its
@@ -734,7 +730,7 @@ struct NearCfg {
     // far (FP64), or an aux item's slip rates (FP64) and one row of B steps for each of its lane groups' slices
     static constexpr size_t warp_bytes(int chunk) {
         const size_t rows = (size_t)((chunk + G - 1) / G * G + B - 1) * pitch * sizeof(R);
-        const size_t win = (rows + 15) / 16 * 16 + (chunk > 16 ? (size_t)B * 32 * 8 : 0);
+        const size_t win = (rows + 15) / 16 * 16 + (chunk > 16 && sizeof(R) == 4 ? (size_t)B * 32 * 8 : 0);
         const size_t aux = (size_t)B * 32 * 8 + (size_t)B * 64 * sizeof(R);
         return ((win > aux ? win : aux) + 15) / 16 * 16;
     }
@@ -749,11 +745,16 @@ struct NearCfg {
 // to four groups; then FP64.  (A uniform slip rate cancels over the sources of a slice, not over the lags of a
 // source.  With V sources x 4 slices of a load in one sum the FP32 march of N = 300 without approximation was
 // 3.0e-7 off; this way it is 2.1e-7, and curved N = 4096 takes 2.23 instead of 2.17 ms per 64 steps.  One sum a
-// slice: 1.9e-7, but 64 sums in registers, 2.43 ms.)
+// slice: 1.9e-7, but 64 sums in registers, 2.43 ms.)  FP64: the even and the odd sources of a slice, slice by
+// slice, over the item.
+// FP64 plans are bound by the FP64 pipe (two multiply-adds a clock and SM; curved N = 1500 4.91 ms per 32 steps, plain march of
+// N = 256 2.59 ms).  Exact products of 62-bit fixed-point numbers on the FP16 tensor cores took 1.11 and
+// 0.51 ms, but cut off what lies below 2^-61 of a leaf's largest coefficient or slip rate: where only quiet
+// sources of a leaf have arrived, a slip rate at 1e-12 of the largest was good to 3e-7.
 // Leaves of at most 16 receivers split the warp into 32 / span lane groups that take slices (window)
 // or aux slices of their own.
 template <class T, class H, int B>
-__global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_kernel(StepArgs<T> a, int warp_bytes) {
+__global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : sizeof(H) == 8 ? 3 : 4) near_block_kernel(StepArgs<T> a, int warp_bytes) {
     using C = NearCfg<H, B>;
     using R = typename C::R;
     using A = typename NearTypes<H>::Aux;
@@ -793,7 +794,7 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
         if (tk.k0 < n + nb) {   // (otherwise the item's window lies before the march)
             R* rows = (R*)mem;
             uint4 xn[G];
-            load(grp, 0, xn);
+            if constexpr (sizeof(R) == 4 || B == 1) load(grp, 0, xn);
             // row q: slip rates of step n + B - 1 - k0 - q (zero before the march, past the steps that
             // the launch may use, and past the item's window)
             {
@@ -814,60 +815,114 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : 4) near_block_ke
             R acc[B];
 #pragma unroll
             for (int b = 0; b < B; ++b) acc[b] = 0;
-            double* mid = (double*)(mem + warp_bytes) - B * 32;   // the sums so far, past 16 slices
-            const R ks = (R)a.kinv;   // the storage scale of the window (FP16), a power of two
             const int iters = (ngr + ngrp - 1) / ngrp;
-            for (int i = 0; i < iters; ++i) {
-                const int gr = i * ngrp + grp;
-                const R* rg = rows + (size_t)min(gr, ngr - 1) * G * P;
-                R s[2][B];   // sums of two slices each over the sources (see above)
+            if constexpr (sizeof(R) == 8) {
+                for (int i = 0; i < iters; ++i) {
+                    const int gr = i * ngrp + grp, left = nk - gr * G;   // slices from the group's first on
+                    const R* rg = rows + (size_t)min(gr, ngr - 1) * G * P;
+                    if constexpr (B == 1) {   // (bound by memory: the group's loads in flight together)
+                        R s[G][2];
 #pragma unroll
-                for (int b = 0; b < B; ++b) s[0][b] = s[1][b] = 0;
-                for (int jb = 0; jb < nbk; ++jb) {
-                    R x[G][V];
+                        for (int g = 0; g < G; ++g) s[g][0] = s[g][1] = 0;
+                        for (int jb = 0; jb < nbk; ++jb) {
+                            R x[G][V];
 #pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        if constexpr (sizeof(H) == 2) unpack(xn[g], x[g], __half());
-                        else unpack(xn[g], x[g], R());
-                    }
-                    const bool wrapj = jb + 1 == nbk;
-                    load(wrapj ? gr + ngrp : gr, wrapj ? 0 : jb + 1, xn);
+                            for (int g = 0; g < G; ++g) unpack(xn[g], x[g], R());
+                            const bool wrapj = jb + 1 == nbk;
+                            load(wrapj ? gr + ngrp : gr, wrapj ? 0 : jb + 1, xn);
 #pragma unroll
-                    for (int q = 0; q < B + G - 1; ++q) {
-                        R y[V];
-                        load_row<V>(rg + q * P + jb * V, y);
+                            for (int g = 0; g < G; ++g) {
+                                R y[V];
+                                load_row<V>(rg + g * P + jb * V, y);
 #pragma unroll
-                        for (int g = 0; g < G; ++g) {
-                            const int b = B - 1 - q + g;
-                            if (b >= 0 && b < B) {
-                                constexpr int U = V < 4 ? V : 4;
-                                R t = x[g][0] * y[0];
-#pragma unroll
-                                for (int v = 1; v < U; ++v) t = fma(x[g][v], y[v], t);
-                                if constexpr (V == 8) {
-                                    R u = x[g][4] * y[4];
-#pragma unroll
-                                    for (int v = 5; v < V; ++v) u = fma(x[g][v], y[v], u);
-                                    t += u;
-                                }
-                                s[g / 2][b] += t;
+                                for (int v = 0; v < 2; ++v) s[g][v] = fma(x[g][v], y[v], s[g][v]);
                             }
+                        }
+#pragma unroll
+                        for (int g = 0; g < G; ++g)
+                            if (g < left) acc[0] += s[g][0] + s[g][1];
+                    } else {
+#pragma unroll 1
+                        for (int g = 0; g < min(G, left); ++g) {
+                            const uint4* c = (const uint4*)(base + (size_t)(gr * G + g) * tk.sl);
+                            uint4 xv = in ? __ldcs(c) : make_uint4(0, 0, 0, 0);
+                            R s[2][B];
+#pragma unroll
+                            for (int b = 0; b < B; ++b) s[0][b] = s[1][b] = 0;
+                            for (int jb = 0; jb < nbk; ++jb) {
+                                R x[V];
+                                unpack(xv, x, R());
+                                if (jb + 1 < nbk && in) xv = __ldcs(c + (size_t)(jb + 1) * nr);
+#pragma unroll
+                                for (int b = 0; b < B; ++b) {
+                                    R y[V];
+                                    load_row<V>(rg + (B - 1 - b + g) * P + jb * V, y);
+#pragma unroll
+                                    for (int v = 0; v < 2; ++v) s[v][b] = fma(x[v], y[v], s[v][b]);
+                                }
+                            }
+#pragma unroll
+                            for (int b = 0; b < B; ++b) acc[b] += s[0][b] + s[1][b];
                         }
                     }
                 }
 #pragma unroll
-                for (int b = 0; b < B; ++b) acc[b] += s[0][b] + s[1][b];
-                if ((i & 3) == 3 && i + 1 < iters) {
+                for (int b = 0; b < B; ++b) tot[b] = acc[b];
+            } else {
+                double* mid = (double*)(mem + warp_bytes) - B * 32;   // the sums so far, past 16 slices
+                const R ks = (R)a.kinv;   // the storage scale of the window (FP16), a power of two
+                for (int i = 0; i < iters; ++i) {
+                    const int gr = i * ngrp + grp;
+                    const R* rg = rows + (size_t)min(gr, ngr - 1) * G * P;
+                    R s[2][B];   // sums of two slices each over the sources (see above)
 #pragma unroll
-                    for (int b = 0; b < B; ++b) {
-                        const double v = wide(acc[b] * ks);
-                        mid[b * 32 + lane] = i > 3 ? mid[b * 32 + lane] + v : v;
-                        acc[b] = 0;
+                    for (int b = 0; b < B; ++b) s[0][b] = s[1][b] = 0;
+                    for (int jb = 0; jb < nbk; ++jb) {
+                        R x[G][V];
+#pragma unroll
+                        for (int g = 0; g < G; ++g) {
+                            if constexpr (sizeof(H) == 2) unpack(xn[g], x[g], __half());
+                            else unpack(xn[g], x[g], R());
+                        }
+                        const bool wrapj = jb + 1 == nbk;
+                        load(wrapj ? gr + ngrp : gr, wrapj ? 0 : jb + 1, xn);
+#pragma unroll
+                        for (int q = 0; q < B + G - 1; ++q) {
+                            R y[V];
+                            load_row<V>(rg + q * P + jb * V, y);
+#pragma unroll
+                            for (int g = 0; g < G; ++g) {
+                                const int b = B - 1 - q + g;
+                                if (b >= 0 && b < B) {
+                                    constexpr int U = V < 4 ? V : 4;
+                                    R t = x[g][0] * y[0];
+#pragma unroll
+                                    for (int v = 1; v < U; ++v) t = fma(x[g][v], y[v], t);
+                                    if constexpr (V == 8) {
+                                        R u = x[g][4] * y[4];
+#pragma unroll
+                                        for (int v = 5; v < V; ++v) u = fma(x[g][v], y[v], u);
+                                        t += u;
+                                    }
+                                    s[g / 2][b] += t;
+                                }
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int b = 0; b < B; ++b) acc[b] += s[0][b] + s[1][b];
+                    if ((i & 3) == 3 && i + 1 < iters) {
+#pragma unroll
+                        for (int b = 0; b < B; ++b) {
+                            const double v = wide(acc[b] * ks);
+                            mid[b * 32 + lane] = i > 3 ? mid[b * 32 + lane] + v : v;
+                            acc[b] = 0;
+                        }
                     }
                 }
-            }
 #pragma unroll
-            for (int b = 0; b < B; ++b) tot[b] = wide(acc[b] * ks) + (iters > 4 ? mid[b * 32 + lane] : 0.0);
+                for (int b = 0; b < B; ++b) tot[b] = wide(acc[b] * ks) + (iters > 4 ? mid[b * 32 + lane] : 0.0);
+            }
         }
     } else if constexpr (sizeof(H) != 2) {   // (those of FP16 plans go to the FP32 instance)
         // aux slices: slice 0 the static tile (times C_j(n - W), it carries dt), slice 1 + q the tail
@@ -1046,8 +1101,8 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
     constexpr int VA = 16 / (int)sizeof(A);
     auto load_x = [&](const RecLeaf& L, int k, uint4 (&x)[NB]) {
         if (k < 0) return;   // (a static tile is read where it is used)
-        const H* sl = (const H*)a.rec_tensor + L.off + (size_t)k * L.sl + (size_t)(lane < L.nr ? lane : 0) * V;
-        const bool in = FDPH_IDX(L.off + (long long)(k + 1) * L.sl <= a.len_rec, a.err);
+        const H* sl = (const H*)a.tensor + L.off + (size_t)k * L.sl + (size_t)(lane < L.nr ? lane : 0) * V;
+        const bool in = FDPH_IDX(L.off + (long long)(k + 1) * L.sl <= a.len_tensor, a.err);
 #pragma unroll
         for (int jb = 0; jb < NB; ++jb)
             x[jb] = in && jb * V < L.ns ? *(const uint4*)(sl + (size_t)jb * L.nr * V) : make_uint4(0, 0, 0, 0);
@@ -1085,8 +1140,8 @@ __global__ void __launch_bounds__(kRupThreads, sizeof(H) == 8 ? 1 : 2) rup_step_
         R s = 0;
         const bool fixed = k < 0;
         if (fixed) {
-            const A* sl = (const A*)(sizeof(H) == 8 ? a.rec_tensor : a.stat) + L.stat + (size_t)(lane < nr ? lane : 0) * VA;
-            const bool in = FDPH_IDX(L.stat + (long long)((ns + VA - 1) / VA) * VA * nr <= (sizeof(H) == 8 ? a.len_rec : a.len_aux), a.err);
+            const A* sl = (const A*)a.stat + L.stat + (size_t)(lane < nr ? lane : 0) * VA;
+            const bool in = FDPH_IDX(L.stat + (long long)((ns + VA - 1) / VA) * VA * nr <= a.len_aux, a.err);
             for (int jb = 0; jb * VA < ns && in; ++jb) {
                 R xv[VA], y[VA];
                 unpack(*(const uint4*)(sl + (size_t)jb * nr * VA), xv, R());

@@ -50,6 +50,6 @@ def _check(prec, u, q):
 
 
 @pytest.mark.parametrize("q", [1e-4, 1e-8, 1e-12])
-@pytest.mark.parametrize("prec,u", [(fdph.FP32, 2.0 ** -20), (fdph.FP16, 2.0 ** -11 + 2.0 ** -20)])
+@pytest.mark.parametrize("prec,u", [(fdph.FP64, 1e-11), (fdph.FP32, 2.0 ** -20), (fdph.FP16, 2.0 ** -11 + 2.0 ** -20)])
 def test_quiet_sources(prec, u, q):
     _check(prec, u, q)
