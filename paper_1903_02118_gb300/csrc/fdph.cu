@@ -60,6 +60,32 @@ __global__ void ring_to_float_kernel(const double* x, float* y, long long n) {
     if (i < n) y[i] = (float)x[i];
 }
 
+// One ring of a saved state.  It is saved with the slots that one step needs (row of step s at s modulo that
+// number), not with the room that a block of steps takes beside them.
+struct RingMap {
+    long long saved, dev;     // first double of the ring as saved and in device memory
+    int rows, room_rows;      // slots as saved and in device memory
+    int width, top;           // doubles of a slot, newest step
+};
+
+// Doubles x0 ... x1 - 1 of the saved form of an array of rings (in order of `saved`), to or from stage[0 ...]
+__global__ void copy_rings_kernel(const RingMap* maps, int n, long long x0, long long x1, double* dev, double* stage,
+                                  bool save) {
+    for (long long x = x0 + (long long)blockIdx.x * blockDim.x + threadIdx.x; x < x1; x += (long long)gridDim.x * blockDim.x) {
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (maps[mid].saved <= x) lo = mid; else hi = mid - 1;
+        }
+        const RingMap g = maps[lo];
+        const int slot = (int)((x - g.saved) / g.width), col = (int)((x - g.saved) % g.width);
+        const int step = g.top - wrap(g.top - slot, g.rows);   // the step of that slot among the newest g.rows
+        double* d = dev + g.dev + (long long)wrap(step, g.room_rows) * g.width + col;
+        if (save) stage[x - x0] = *d;
+        else *d = stage[x - x0];
+    }
+}
+
 // Bounded mbarrier wait (PTX)
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -329,6 +355,7 @@ struct fdph_plan_s {
     double kscale = 1.0;      // FP16 window coefficients are stored as K * kscale (a power of two)
     int sched_version = 0;    // bumped whenever the near-field items are rebuilt
     size_t partial_cap = 0;   // capacity of `partial`, in doubles
+    RingMap* maps = nullptr;  // rings of the array being saved or restored
     // branches of a step that run concurrently with the near field: [0] FIR + scatter,
     // [1] transient convolution + Eq. 39 evaluation (fork after push, join before gather)
     cudaStream_t side[2] = {nullptr, nullptr};
@@ -2122,18 +2149,12 @@ int fdph_get_stats(fdph_plan_t P, fdph_stats* s) {
     return FDPH_OK;
 }
 
-// The arrays of a saved state.  Rings are saved with the slots that one step needs (row of step s at
-// s modulo that length), not with the room that a block of steps takes beside them.
+// The arrays of a state saved at step n (n < 0: their sizes only)
 struct StateArray {
     double* p;
     size_t count;                 // doubles of one right-hand side as saved
     size_t stored;                // doubles of one right-hand side in device memory
-    // rings: (saved rows, device rows, doubles per row, newest step, first double saved, stored)
-    struct Ring {
-        int rows, room_rows, width, top;
-        size_t save_at, at;
-    };
-    std::vector<Ring> rings;
+    std::vector<RingMap> rings;
 };
 
 static std::vector<StateArray> state_arrays(fdph_plan_t P, int n) {
@@ -2141,9 +2162,7 @@ static std::vector<StateArray> state_arrays(fdph_plan_t P, int n) {
     std::vector<StateArray> v;
     auto ring1 = [&](double* p, int rows_dev) {
         const int rows = rows_dev - kRingRoom;
-        StateArray a{p, (size_t)rows * P->N, (size_t)rows_dev * P->N, {}};
-        a.rings.push_back({rows, rows_dev, P->N, n - 1, 0, 0});
-        v.push_back(a);
+        v.push_back({p, (size_t)rows * P->N, (size_t)rows_dev * P->N, {{0, 0, rows, rows_dev, P->N, n - 1}}});
     };
     auto plain = [&](double* p, size_t c) { v.push_back({p, c, std::max<size_t>(c, 1), {}}); };
     ring1(P->Dring, P->WD);
@@ -2152,35 +2171,60 @@ static std::vector<StateArray> state_arrays(fdph_plan_t P, int n) {
     plain(P->Ccomp, P->N);
     StateArray r{P->ring, 0, (size_t)std::max<int64_t>(hp.ring_len, 1), {}}, z{P->zring, 0, (size_t)std::max<int64_t>(hp.zring_len, 1), {}};
     for (const SubBlock& b : hp.sbs) {
-        r.rings.push_back({b.L - kRingRoom, b.L, b.rank, n - 1 + b.maxdelay, r.count, (size_t)b.ring});
+        if (!b.rank) continue;
+        if (n >= 0) r.rings.push_back({(long long)r.count, (long long)b.ring, b.L - kRingRoom, b.L, b.rank, n - 1 + b.maxdelay});
         r.count += (size_t)(b.L - kRingRoom) * b.rank;
         if (b.kind != SB_TR) continue;
-        z.rings.push_back({b.LZ - kRingRoom, b.LZ, b.rank, n - 1 - b.mindm, z.count, (size_t)b.zring});
+        if (n >= 0) z.rings.push_back({(long long)z.count, (long long)b.zring, b.LZ - kRingRoom, b.LZ, b.rank, n - 1 - b.mindm});
         z.count += (size_t)(b.LZ - kRingRoom) * b.rank;
     }
-    v.push_back(r);
-    v.push_back(z);
+    v.push_back(std::move(r));
+    v.push_back(std::move(z));
     plain(P->ustate, (size_t)hp.ustate_len);
     plain(P->vstate, (size_t)hp.vstate_len);
     plain(P->uhist, (size_t)P->uhist_len);
     return v;
 }
 
-// the rows of the newest steps between a saved ring and a device ring (host copies)
-static void copy_ring(const StateArray::Ring& g, double* saved, double* dev, bool save) {
-    auto slot = [](long long s, int L) { return (size_t)((s % L + L) % L); };
-    for (long long s = (long long)g.top - g.rows + 1; s <= g.top; ++s) {
-        double* a = saved + g.save_at + slot(s, g.rows) * g.width;
-        double* b = dev + g.at + slot(s, g.room_rows) * g.width;
-        if (save) memcpy(a, b, g.width * sizeof(double));
-        else memcpy(b, a, g.width * sizeof(double));
+// An array's saved form [nrhs][count] to or from host memory.  Rings are re-arranged on the device, staged
+// in the partial sums (scratch of a block of steps, of which none is under way).
+static int copy_state_array(fdph_plan_t P, const StateArray& a, char* host, bool save) {
+    cudaStream_t s = P->stream;
+    if (!a.count) return FDPH_OK;
+    if (!save) FDPH_CUDA(cudaMemsetAsync(a.p, 0, a.stored * P->nrhs * sizeof(double), s));
+    if (!a.rings.empty()) {
+        if (!P->maps) {   // (the far rings are the most)
+            int rc = dalloc(P, &P->maps, std::max<size_t>(P->hp.sbs.size(), 1));
+            if (rc) return rc;
+        }
+        FDPH_CUDA(cudaMemcpyAsync(P->maps, a.rings.data(), a.rings.size() * sizeof(RingMap), cudaMemcpyHostToDevice, s));
     }
+    const long long cap = (long long)P->partial_cap * kBlk * P->nrhs;
+    for (int q = 0; q < P->nrhs; ++q) {
+        char* h = host + q * a.count * sizeof(double);
+        double* d = a.p + q * a.stored;
+        if (a.rings.empty()) {
+            FDPH_CUDA(cudaMemcpyAsync(save ? (void*)h : (void*)d, save ? (void*)d : (void*)h, a.count * sizeof(double),
+                                      save ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, s));
+            continue;
+        }
+        for (long long x0 = 0; x0 < (long long)a.count; x0 += cap) {
+            const long long x1 = std::min<long long>(a.count, x0 + cap);
+            const size_t bytes = (size_t)(x1 - x0) * sizeof(double);
+            if (!save) FDPH_CUDA(cudaMemcpyAsync(P->partial, h + x0 * sizeof(double), bytes, cudaMemcpyHostToDevice, s));
+            copy_rings_kernel<<<(int)std::min<long long>(blocks(x1 - x0, 256), 152 * 8), 256, 0, s>>>(
+                P->maps, (int)a.rings.size(), x0, x1, d, P->partial, save);
+            FDPH_CUDA(cudaGetLastError());
+            if (save) FDPH_CUDA(cudaMemcpyAsync(h + x0 * sizeof(double), P->partial, bytes, cudaMemcpyDeviceToHost, s));
+        }
+    }
+    return FDPH_OK;
 }
 
 int fdph_save_state(fdph_plan_t P, void* buf, size_t* len) {
     if (!P || !len) return FDPH_E_ARG;
     if (P->predicted) return pending_commit(P);
-    const std::vector<StateArray> arrays = state_arrays(P, P->n);
+    const std::vector<StateArray> arrays = state_arrays(P, buf ? P->n : -1);
     size_t need = sizeof(int32_t) * 2;
     for (const StateArray& a : arrays) need += a.count * P->nrhs * sizeof(double);
     if (P->rupture) need += (size_t)P->N * sizeof(double);   // the friction law's accumulated slip
@@ -2194,29 +2238,16 @@ int fdph_save_state(fdph_plan_t P, void* buf, size_t* len) {
     int32_t hdr[2] = {P->n, P->N};
     memcpy(o, hdr, sizeof(hdr));
     o += sizeof(hdr);
-    std::vector<double> dev, saved;
     for (const StateArray& a : arrays) {   // [nrhs][count] (a zero count stays empty)
-        if (a.count) {
-            dev.resize(a.stored * P->nrhs);
-            FDPH_CUDA(cudaMemcpyAsync(dev.data(), a.p, dev.size() * sizeof(double), cudaMemcpyDeviceToHost, P->stream));
-            FDPH_CUDA(cudaStreamSynchronize(P->stream));
-            for (int q = 0; q < P->nrhs; ++q) {
-                double* src = dev.data() + q * a.stored;
-                if (a.rings.empty()) {
-                    memcpy(o + q * a.count * sizeof(double), src, a.count * sizeof(double));
-                    continue;
-                }
-                saved.assign(a.count, 0.0);
-                for (const auto& g : a.rings) copy_ring(g, saved.data(), src, true);
-                memcpy(o + q * a.count * sizeof(double), saved.data(), a.count * sizeof(double));
-            }
+        int rc = copy_state_array(P, a, o, true);
+        if (rc) {
+            cudaStreamSynchronize(P->stream);   // (no copy into the caller's buffer stays in flight)
+            return rc;
         }
         o += a.count * P->nrhs * sizeof(double);
     }
-    if (P->rupture) {
-        FDPH_CUDA(cudaMemcpyAsync(o, P->fr.slip, P->N * sizeof(double), cudaMemcpyDeviceToHost, P->stream));
-        FDPH_CUDA(cudaStreamSynchronize(P->stream));   // the caller's buffer is complete on return
-    }
+    if (P->rupture) FDPH_CUDA(cudaMemcpyAsync(o, P->fr.slip, P->N * sizeof(double), cudaMemcpyDeviceToHost, P->stream));
+    FDPH_CUDA(cudaStreamSynchronize(P->stream));   // the caller's buffer is complete on return
     *len = need;
     return FDPH_OK;
 }
@@ -2240,22 +2271,11 @@ int fdph_load_state(fdph_plan_t P, const void* buf, size_t len) {
     }
     o += sizeof(hdr);
     FDPH_CUDA(cudaStreamSynchronize(P->stream));
-    std::vector<double> dev, saved;
-    for (const StateArray& a : state_arrays(P, hdr[0])) {
-        if (a.count) {
-            dev.assign(a.stored * P->nrhs, 0.0);
-            for (int q = 0; q < P->nrhs; ++q) {
-                const char* src = o + q * a.count * sizeof(double);
-                if (a.rings.empty()) {
-                    memcpy(dev.data() + q * a.stored, src, a.count * sizeof(double));
-                    continue;
-                }
-                saved.resize(a.count);
-                memcpy(saved.data(), src, a.count * sizeof(double));
-                for (const auto& g : a.rings) copy_ring(g, saved.data(), dev.data() + q * a.stored, false);
-            }
-            FDPH_CUDA(cudaMemcpyAsync(a.p, dev.data(), dev.size() * sizeof(double), cudaMemcpyHostToDevice, P->stream));
-            FDPH_CUDA(cudaStreamSynchronize(P->stream));
+    const std::vector<StateArray> arrays = state_arrays(P, hdr[0]);   // (read by copies in flight)
+    for (const StateArray& a : arrays) {
+        if ((rc = copy_state_array(P, a, const_cast<char*>(o), false))) {
+            cudaStreamSynchronize(P->stream);
+            return rc;
         }
         o += a.count * P->nrhs * sizeof(double);
     }
