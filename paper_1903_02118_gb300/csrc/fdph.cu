@@ -834,7 +834,8 @@ static int run_host(fdph_plan_t P, int steps, const double* D_host, double* T_ho
     FDPH_CUDA(cudaStreamSynchronize(P->stream));
     FDPH_CUDA(cudaStreamSynchronize(P->d2h));
     cudaError_t e = cudaSuccess;
-    for (int k = 0, i = 0; k < steps && e == cudaSuccess; ++i) {
+    int rc = FDPH_OK;
+    for (int k = 0, i = 0; k < steps && e == cudaSuccess && !rc; ++i) {
         const int q = i % S, nb = std::min(kBlk, steps - k);
         double *dD = P->io_D + q * kBlk * row, *dT = P->io_T + q * kBlk * row;
         if (i >= S) e = cudaStreamWaitEvent(P->h2d, P->ev_free[q], 0);
@@ -842,9 +843,7 @@ static int run_host(fdph_plan_t P, int steps, const double* D_host, double* T_ho
             e = cudaMemcpyAsync(dD, D_host + k * row, nb * row * sizeof(double), cudaMemcpyHostToDevice, P->h2d);
         if (e == cudaSuccess) e = cudaEventRecord(P->ev_in[q], P->h2d);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(P->stream, P->ev_in[q], 0);
-        if (e != cudaSuccess) break;
-        int rc = run_any(P, nb, dD, dT);
-        if (rc) return rc;
+        if (e != cudaSuccess || (rc = run_any(P, nb, dD, dT))) break;
         e = cudaEventRecord(P->ev_out[q], P->stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(P->d2h, P->ev_out[q], 0);
         if (e == cudaSuccess)
@@ -852,8 +851,12 @@ static int run_host(fdph_plan_t P, int steps, const double* D_host, double* T_ho
         if (e == cudaSuccess) e = cudaEventRecord(P->ev_free[q], P->d2h);
         k += nb;
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(P->d2h);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(P->stream);
+    // no copy from or to the caller's buffers stays in flight, after an error either
+    for (cudaStream_t s : {P->h2d, P->stream, P->d2h}) {
+        const cudaError_t w = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = w;
+    }
+    if (rc) return rc;
     if (e != cudaSuccess) {
         set_error(std::string("fdph_run_host: ") + cudaGetErrorString(e));
         return FDPH_E_CUDA;
