@@ -524,13 +524,29 @@ struct ProfScope {
 
 // The kernels hold one column per step of a launch in registers: instantiated for one step and for a
 // whole block (a shorter block computes unused columns)
+// (one step of several right-hand sides: all of them in one lane of the FIR and the scatter)
+template <class T, int NR>
+static void launch_fir_step(const StepArgs<T>& a, cudaStream_t s) {
+    const size_t smem = (size_t)kFirWarps * NR * (a.fir_taps + 2) * sizeof(T);
+    const bool staged = smem <= 48 * 1024;   // (no opt-in shared memory)
+    fir_step_kernel<T, NR><<<blocks(a.n_fir, kFirWarps * kFirGroups), 32 * kFirWarps, staged ? smem : 0, s>>>(a, staged);
+}
+
 template <class T>
 static void launch_fir(const StepArgs<T>& a, cudaStream_t s) {
+    if (a.nb == 1) {
+        switch (a.nrhs) {
+            case 2: launch_fir_step<T, 2>(a, s); break;
+            case 4: launch_fir_step<T, 4>(a, s); break;
+            case 8: launch_fir_step<T, 8>(a, s); break;
+            default: launch_fir_step<T, 1>(a, s);
+        }
+        return;
+    }
     const dim3 g(blocks(a.n_fir, kFirWarps), a.nrhs);
-    const size_t smem = (size_t)kFirWarps * (a.fir_taps + 2 * (a.nb == 1 ? 1 : kBlk)) * sizeof(T);
-    const bool staged = smem <= 48 * 1024;   // (no opt-in shared memory)
-    if (a.nb == 1) fir_kernel<T, 1><<<g, 32 * kFirWarps, staged ? smem : 0, s>>>(a, staged);
-    else fir_kernel<T, kBlk><<<g, 32 * kFirWarps, staged ? smem : 0, s>>>(a, staged);
+    const size_t smem = (size_t)kFirWarps * (a.fir_taps + 2 * kBlk) * sizeof(T);
+    const bool staged = smem <= 48 * 1024;
+    fir_kernel<T, kBlk><<<g, 32 * kFirWarps, staged ? smem : 0, s>>>(a, staged);
 }
 
 // Eq. 42: scatter into the delay rings, or (far_mode 1, one step) record the source values and gather
@@ -541,7 +557,13 @@ static void launch_eq42(const StepArgs<T>& a, cudaStream_t s) {
         record_kernel<T><<<dim3(blocks(a.n_rec, 128), a.nrhs), 128, 0, s>>>(a);
         if (a.n_gat) hgather_kernel<T><<<dim3(blocks((long long)a.n_gat * 32, 128), a.nrhs), 128, 0, s>>>(a);
     } else if (a.n_sct) {
-        scatter_kernel<T><<<dim3(blocks((long long)a.n_sct * 32, 128), a.nrhs), 128, 0, s>>>(a);
+        const int g = blocks((long long)a.n_sct * 32, 128);
+        switch (a.nb == 1 ? a.nrhs : 1) {
+            case 2: scatter_kernel<T, 2><<<g, 128, 0, s>>>(a); break;
+            case 4: scatter_kernel<T, 4><<<g, 128, 0, s>>>(a); break;
+            case 8: scatter_kernel<T, 8><<<g, 128, 0, s>>>(a); break;
+            default: scatter_kernel<T, 1><<<dim3(g, a.nrhs), 128, 0, s>>>(a);
+        }
     }
 }
 
@@ -572,9 +594,10 @@ static void launch_near_items(const StepArgs<T>& a, int chunk, cudaStream_t s) {
 }
 
 // the tensor-core window items
-template <int NR, int B>
+template <int NR>
 static void launch_tc(const StepArgs<float>& a, int n_win, int chunk, cudaStream_t s) {
-    tc_block_kernel<NR, B><<<n_win, 32 * TcCfg<NR, B>::warps, TcCfg<NR, B>::smem(chunk), s>>>(a, chunk);
+    if (a.nb == 1) tc_step_kernel<NR><<<blocks(n_win, kTcStepWarps), 32 * kTcStepWarps, 0, s>>>(a, n_win);
+    else tc_block_kernel<NR><<<n_win, 32 * TcCfg<NR>::warps, TcCfg<NR>::smem(chunk), s>>>(a, chunk);
 }
 
 // The near field of a launch: the window items (FP16 plans), or all items (FP64 and FP32 plans).  FP16 windows of
@@ -589,14 +612,13 @@ static void launch_near(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
         else launch_near_items<T, double, kBlk>(a, P->chunk, s);
     } else if (P->precision == FDPH_FP16) {
         if (!P->n_win) return;
-        const bool one = a.nb == 1;
-        StepArgs<T> w = a;   // (one right-hand side)
+        StepArgs<T> w = a;   // (a block of one right-hand side)
         w.n_items = P->n_win;
         switch (P->nrhs) {
-            case 2: one ? launch_tc<2, 1>(a, P->n_win, P->chunk, s) : launch_tc<2, kBlk>(a, P->n_win, P->chunk, s); break;
-            case 4: one ? launch_tc<4, 1>(a, P->n_win, P->chunk, s) : launch_tc<4, kBlk>(a, P->n_win, P->chunk, s); break;
-            case 8: one ? launch_tc<8, 1>(a, P->n_win, P->chunk, s) : launch_tc<8, kBlk>(a, P->n_win, P->chunk, s); break;
-            default: one ? launch_near_items<T, __half, 1>(w, P->chunk, s) : launch_near_items<T, __half, kBlk>(w, P->chunk, s);
+            case 2: launch_tc<2>(a, P->n_win, P->chunk, s); break;
+            case 4: launch_tc<4>(a, P->n_win, P->chunk, s); break;
+            case 8: launch_tc<8>(a, P->n_win, P->chunk, s); break;
+            default: a.nb == 1 ? launch_near_items<T, __half, 1>(a, P->chunk, s) : launch_near_items<T, __half, kBlk>(w, P->chunk, s);
         }
     } else if (a.nb == 1) {
         launch_near_items<T, float, 1>(a, P->chunk, s);
@@ -606,11 +628,12 @@ static void launch_near(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
 }
 
 // The static and tail items of FP16 plans: a kernel of their own, far from filling the GPU, so it goes last
-// on the far-field branch, beside the windows
+// on the far-field branch, beside the windows.  (A single step of one right-hand side takes them along with its
+// windows: nothing there is as long as one more kernel on that branch; N = 400, leaves of 13, 43 -> 32 us.)
 template <class T>
 static void launch_near_aux(fdph_plan_t P, StepArgs<T> a, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
-        if (P->precision != FDPH_FP16 || !P->n_aux) return;
+        if (P->precision != FDPH_FP16 || !P->n_aux || (a.nb == 1 && P->nrhs == 1)) return;
         a.tasks += P->n_win;
         a.n_items = P->n_aux;
         if (a.nb == 1) launch_near_items<T, float, 1>(a, P->chunk, s);
@@ -780,6 +803,16 @@ static void drop_graphs(fdph_plan_t P) {
     P->graphs.clear();
 }
 
+// The longest run of steps that is cheaper step by step than as a block, whose kernels take (nearly) as long for two steps
+// as for sixteen.  us, step / block of 2, 3, 5: FP64 N = 1500 193 / 698, 830, 1125, eight right-hand sides of N = 400
+// 282 / 978, 1168, 1606; FP16 N = 6000, eight 516 / 2704, 2822, four 375 / 1525, 1576; FP32 N = 1500, eight 347 / 973, four
+// 188 / 482; one FP16 with 16 tail terms, N = 1500, 81 / 248, 257; one FP32 without 77 / 163, N = 400 30 / 52.
+static int stepwise(fdph_plan_t P) {
+    if (P->precision == FDPH_FP64) return 4;
+    if (P->precision == FDPH_FP16) return P->nrhs < 4 ? 2 : 3;
+    return P->nrhs >= 4 || P->hp.soe > 0 ? 2 : 1;
+}
+
 // `steps` steps with given slip rates, in blocks.  A caller may pass D == T (every block reads its rows
 // before it writes them) but rows that overlap otherwise are taken one step at a time, as is the
 // delayed-history form, whose steps replay a graph.
@@ -800,7 +833,7 @@ static int run_steps(fdph_plan_t P, int steps, const double* D, double* Tout) {
     }
     while (k < steps) {
         StepArgs<T> a = make_args<T>(P, D + k * row, Tout + k * row);
-        a.nb = alias || P->n_rec ? 1 : std::min(kBlk, steps - k);
+        a.nb = alias || P->n_rec || steps - k <= stepwise(P) ? 1 : std::min(kBlk, steps - k);
         enqueue_block<T>(P, a, P->stream);
         FDPH_CUDA(cudaGetLastError());
         P->n += a.nb;
@@ -1004,12 +1037,9 @@ static int build_schedule(fdph_plan_t P) {
                                        (int)NearCfg<H, 1>::warp_bytes(kChunk) * kNearWarps));
         FDPH_CUDA(cudaFuncSetAttribute(near_block_kernel<T, H, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)NearCfg<H, kBlk>::warp_bytes(kChunk) * kNearWarps));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<2, 1>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<2, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<2, kBlk>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<4, 1>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<4, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<4, kBlk>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8, 1>::smem(kChunk)));
-        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8, kBlk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8, kBlk>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<2>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<4>::smem(kChunk)));
+        FDPH_CUDA(cudaFuncSetAttribute(tc_block_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<8>::smem(kChunk)));
     }
     constexpr int longest = sizeof(H) == 8 ? kChunk : 2 * kChunk;   // (near_max_chunk)
     using I = typename std::conditional<sizeof(H) == 8, double, float>::type;

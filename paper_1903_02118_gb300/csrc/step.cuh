@@ -121,7 +121,7 @@ struct StepArgs {
     double* Cring;            // [WC][N]
     double* C;                // [N] cumulative slip (rounded sum)
     double* Ccomp;            // [N] Kahan compensation
-    double *blkD, *blkC;      // [N][kBlk] D and dt C of the block's steps
+    double *blkD, *blkC;      // D and dt C of the block's steps, [N][kBlk]; of one step [N][nrhs] (blk_pitch)
     // far field
     const SbDev* sbs;
     const T* fac;
@@ -145,7 +145,7 @@ struct StepArgs {
     int n_tr;
     double* ring;
     double* zring;
-    T* dhat;                  // [tasks][kBlk]
+    T* dhat;                  // [tasks][kBlk]; of one step [tasks][nrhs]
     long long len_ring, len_zring, len_dhat, len_ustate, len_vstate;
     // near field
     const NearTask* tasks;    // near-field work items, largest first
@@ -204,6 +204,13 @@ __device__ __forceinline__ int hist_end(const StepArgs<T>& a, int n) {
     return a.hist == HIST_ALL ? n + a.nb : a.hist == HIST_BASE ? (n & ~(kBlk - 1)) : n;
 }
 
+// pitch of blkD, blkC and dhat (scratch of one launch sequence): the steps of a block side by side, or the
+// right-hand sides of a single step, so that the scatter reads them together
+template <class T>
+__device__ __forceinline__ int blk_pitch(const StepArgs<T>& a) {
+    return a.nb == 1 ? a.nrhs : kBlk;
+}
+
 // the arguments of right-hand side r
 template <class T>
 __device__ __forceinline__ StepArgs<T> rhs_args(const StepArgs<T>& a0, int r) {
@@ -217,11 +224,11 @@ __device__ __forceinline__ StepArgs<T> rhs_args(const StepArgs<T>& a0, int r) {
         a.Cring = a0.Cring + r * a0.rs_C;
         a.C = a0.C + rN;
         a.Ccomp = a0.Ccomp + rN;
-        a.blkD = a0.blkD + rN * kBlk;
-        a.blkC = a0.blkC + rN * kBlk;
+        a.blkD = a0.blkD + (a0.nb == 1 ? r : rN * kBlk);
+        a.blkC = a0.blkC + (a0.nb == 1 ? r : rN * kBlk);
         a.ring = a0.ring + r * a0.len_ring;
         a.zring = a0.zring + r * a0.len_zring;
-        a.dhat = a0.dhat + r * a0.len_dhat;
+        a.dhat = a0.dhat + (a0.nb == 1 ? r : r * a0.len_dhat);
         a.tfar = a0.tfar + rN * kBlk;
         if (a0.ustate) a.ustate = a0.ustate + r * a0.len_ustate;
         if (a0.vstate) a.vstate = a0.vstate + r * a0.len_vstate;
@@ -303,14 +310,15 @@ __device__ __forceinline__ void push_one(const StepArgs<T>& a, int p, int n, int
     const size_t slot = (size_t)wrap(n, a.WD) * a.N + p;
     a.Dring[slot] = d;
     if (a.Dring32) a.Dring32[slot] = (float)d;
-    a.blkD[(size_t)p * kBlk + b] = d;
+    const size_t at = (size_t)p * blk_pitch(a) + b;
+    a.blkD[at] = d;
     // compensated running sum of the slip (units of dt)
     const double y = d - comp;
     const double t = c + y;
     comp = (t - c) - y;
     c = t;
     a.Cring[(size_t)wrap(n, a.WC) * a.N + p] = t;
-    a.blkC[(size_t)p * kBlk + b] = a.dt * t;
+    a.blkC[at] = a.dt * t;
 }
 
 template <class T>
@@ -373,32 +381,23 @@ __global__ void __launch_bounds__(32 * kFirWarps) fir_kernel(StepArgs<T> a0, boo
     T s0[B], s1[B];
 #pragma unroll
     for (int b = 0; b < B; ++b) s0[b] = s1[b] = 0;
-    // even and odd taps in separate sums
-    if constexpr (B == 1) {
-        int m = 0;
-        for (; m + 1 < g.taps; m += 2) {
-            s0[0] = fma(h[(size_t)m * 32], d_at(m), s0[0]);
-            s1[0] = fma(h[(size_t)(m + 1) * 32], d_at(m + 1), s1[0]);
-        }
-        if (m < g.taps) s0[0] = fma(h[(size_t)m * 32], d_at(m), s0[0]);
-    } else {
-        // taps in chunks of B: the 2 B - 1 slip rates that B taps of B steps need sit in registers
-        for (int m0 = 0; m0 < g.taps; m0 += B) {
-            T x[2 * B - 1];
+    // even and odd taps in separate sums; taps in chunks of B: the 2 B - 1 slip rates that B taps of B steps need
+    // sit in registers
+    for (int m0 = 0; m0 < g.taps; m0 += B) {
+        T x[2 * B - 1];
 #pragma unroll
-            for (int q = 0; q < 2 * B - 1; ++q) x[q] = d_at(min(m0 + q, rows + B - 1));
-            constexpr int F = sizeof(T) == 4 ? B : B / 4;   // taps in flight together (registers)
+        for (int q = 0; q < 2 * B - 1; ++q) x[q] = d_at(min(m0 + q, rows + B - 1));
+        constexpr int F = sizeof(T) == 4 ? B : B / 4;   // taps in flight together (registers)
 #pragma unroll
-            for (int v = 0; v < B; v += F) {
-                T hm[F];
+        for (int v = 0; v < B; v += F) {
+            T hm[F];
 #pragma unroll
-                for (int u = 0; u < F; ++u) hm[u] = m0 + v + u < g.taps ? h[(size_t)(m0 + v + u) * 32] : (T)0;
+            for (int u = 0; u < F; ++u) hm[u] = m0 + v + u < g.taps ? h[(size_t)(m0 + v + u) * 32] : (T)0;
 #pragma unroll
-                for (int u = 0; u < F; ++u)
+            for (int u = 0; u < F; ++u)
 #pragma unroll
-                    for (int b = 0; b < B; ++b)
-                        (u & 1 ? s1 : s0)[b] = fma(hm[u], x[B - 1 - b + v + u], (u & 1 ? s1 : s0)[b]);
-            }
+                for (int b = 0; b < B; ++b)
+                    (u & 1 ? s1 : s0)[b] = fma(hm[u], x[B - 1 - b + v + u], (u & 1 ? s1 : s0)[b]);
         }
     }
     if (lane < g.count) {
@@ -410,14 +409,75 @@ __global__ void __launch_bounds__(32 * kFirWarps) fir_kernel(StepArgs<T> a0, boo
     }
 }
 
+// One step of NR right-hand sides (the sums of fir_kernel): a tap is read once for all of them.  With a grid row per
+// right-hand side every waveform, factor and run was read eight times: eight right-hand sides of N = 6000, one step
+// 98 us here and 395 us in the scatter, now 55 and 133.
+constexpr int kFirGroups = 2;   // groups of a warp, one after the other: mostly of one source, staged once
+
+template <class T, int NR>
+__global__ void __launch_bounds__(32 * kFirWarps) fir_step_kernel(StepArgs<T> a, bool staged) {
+    extern __shared__ __align__(8) unsigned char fir_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n = step_index(a);
+    const int pitch = a.fir_taps + 2;
+    T* sd = (T*)fir_smem + (size_t)warp * NR * pitch;
+    int src = -1;
+    for (int i = 0; i < kFirGroups; ++i) {
+        const int w = (blockIdx.x * kFirWarps + warp) * kFirGroups + i;
+        if (w >= a.n_fir) return;   // warp-uniform
+        const FirGroup g = a.fir[w];
+        if (!FDPH_IDX(g.taps <= a.fir_taps && g.taps <= a.WD && g.src < a.N, a.err)) continue;
+        auto rate = [&](int x, int r) {
+            const int t = n - x;
+            return t >= 0 ? fir_ring(a)[r * a.rs_D + (size_t)wrap(t, a.WD) * a.N + g.src] : (T)0;
+        };
+        if (staged && g.src != src) {
+            __syncwarp();
+            for (int x = lane; x < a.fir_taps; x += 32)
+#pragma unroll
+                for (int r = 0; r < NR; ++r) sd[r * pitch + x] = rate(x, r);
+            __syncwarp();
+            src = g.src;
+        }
+        auto d_at = [&](int x, int r) { return staged ? sd[r * pitch + x] : rate(x, r); };
+        const T* h = a.fir_h + g.h + lane;
+        T s0[NR], s1[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) s0[r] = s1[r] = 0;
+        int m = 0;
+#pragma unroll 4
+        for (; m + 1 < g.taps; m += 2) {
+            const T h0 = h[(size_t)m * 32], h1 = h[(size_t)(m + 1) * 32];
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                s0[r] = fma(h0, d_at(m, r), s0[r]);
+                s1[r] = fma(h1, d_at(m + 1, r), s1[r]);
+            }
+        }
+        if (m < g.taps) {
+            const T h0 = h[(size_t)m * 32];
+#pragma unroll
+            for (int r = 0; r < NR; ++r) s0[r] = fma(h0, d_at(m, r), s0[r]);
+        }
+        if (lane < g.count) {
+            const long long q = a.fir_dhat[g.first + lane];
+            if (FDPH_IDX((q + 1) * kBlk <= a.len_dhat, a.err)) {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) a.dhat[q * NR + r] = s0[r] + s1[r];
+            }
+        }
+    }
+}
+
 // ---- Eq. 42
 
 // source quantity u_j of Eq. 42 of the block's b-th step: Dhat (Domain F), dt * cumulative slip
-// (Domain S, App. B.1), slip rate (transient)
+// (Domain S, App. B.1), slip rate (transient); of a single step, of right-hand side r past the arguments' own
 template <class T>
-__device__ __forceinline__ double source_value(const StepArgs<T>& a, const SbDev& sb, int jl, int b) {
-    if (sb.kind == 0) return wide(a.dhat[(sb.dhat + jl) * kBlk + b]);
-    return (sb.kind == 1 ? a.blkC : a.blkD)[(size_t)(sb.s0 + jl) * kBlk + b];
+__device__ __forceinline__ double source_value(const StepArgs<T>& a, const SbDev& sb, int jl, int b, int r = 0) {
+    const int pitch = blk_pitch(a);
+    if (sb.kind == 0) return wide(a.dhat[(sb.dhat + jl) * pitch + b + r]);
+    return (sb.kind == 1 ? a.blkC : a.blkD)[(size_t)(sb.s0 + jl) * pitch + b + r];
 }
 
 // Eq. 42 slot by slot: the steps of a block add to the ring slots n + mindelay ... n + nb - 1 +
@@ -425,7 +485,8 @@ __device__ __forceinline__ double source_value(const StepArgs<T>& a, const SbDev
 // brings one of the block's steps there, oldest step first.  2^lg lanes per slot cover the rank
 // index, so the slots of a warp are one contiguous piece of the ring, read and written once per
 // block (a step-by-step scatter updates a slot once for every source).
-template <class T>
+// NR right-hand sides in one lane (one step: the factors are read once), or one per grid row (blocks).
+template <class T, int NR>
 __global__ void scatter_kernel(StepArgs<T> a0) {
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const StepArgs<T> a = rhs_args(a0, blockIdx.y);
@@ -441,7 +502,7 @@ __global__ void scatter_kernel(StepArgs<T> a0) {
     const int4 top = a.runs[run];
     if (d - top.x >= nb) return;   // no step of the block comes to this slot
     const int slot = wrap(n + d, sb.L);
-    double* r = a.ring + sb.ring + (long long)slot * rank;
+    double* ring = a.ring + sb.ring + (long long)slot * rank;
     if (!FDPH_IDX(sb.ring + (long long)(slot + 1) * rank <= a.len_ring, a.err)) return;
     if (sb.ident == 2) {
         // G is the identity: column j of a slot receives source j only, once
@@ -451,7 +512,9 @@ __global__ void scatter_kernel(StepArgs<T> a0) {
             if (b >= nb) break;
             for (int u = lj; u < rn.y; u += G) {
                 const int jl = a.src_order[rn.z + u];
-                if (FDPH_IDX(jl < rank, a.err)) r[jl] = source_value(a, sb, jl, b);
+                if (!FDPH_IDX(jl < rank, a.err)) continue;
+#pragma unroll
+                for (int r = 0; r < NR; ++r) ring[r * a.len_ring + jl] = source_value(a, sb, jl, b, r);
             }
         }
         return;
@@ -459,23 +522,33 @@ __global__ void scatter_kernel(StepArgs<T> a0) {
     const bool fresh = d >= maxdelay;   // the slot comes into the ring's range within this block
     const T* g = a.fac + sb.g;
     for (int l = lj; l < rank; l += G) {
-        double v = fresh ? 0.0 : r[l];
+        double v[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) v[r] = fresh ? 0.0 : ring[r * a.len_ring + l];
         for (int q = run; q >= run0; --q) {
             const int4 rn = a.runs[q];
             const int b = d - rn.x;
             if (b >= nb) break;
             if (rn.y == 1) {
-                v = fma(wide(g[(long long)rn.w * rank + l]), source_value(a, sb, rn.w, b), v);
+                const double gl = wide(g[(long long)rn.w * rank + l]);
+#pragma unroll
+                for (int r = 0; r < NR; ++r) v[r] = fma(gl, source_value(a, sb, rn.w, b, r), v[r]);
             } else {
-                double s = 0.0;
+                double s[NR];
+#pragma unroll
+                for (int r = 0; r < NR; ++r) s[r] = 0.0;
                 for (int u = 0; u < rn.y; ++u) {
                     const int jl = a.src_order[rn.z + u];
-                    s = fma(wide(g[(long long)jl * rank + l]), source_value(a, sb, jl, b), s);
+                    const double gl = wide(g[(long long)jl * rank + l]);
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) s[r] = fma(gl, source_value(a, sb, jl, b, r), s[r]);
                 }
-                v += s;
+#pragma unroll
+                for (int r = 0; r < NR; ++r) v[r] += s[r];
             }
         }
-        r[l] = v;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) ring[r * a.len_ring + l] = v[r];
     }
 }
 
@@ -855,6 +928,7 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : sizeof(H) == 8 ?
                                 if (jb + 1 < nbk && in) xv = __ldcs(c + (size_t)(jb + 1) * nr);
 #pragma unroll
                                 for (int b = 0; b < B; ++b) {
+                                    if (b >= nb) break;   // (the launch's steps only: the FP64 pipe bounds)
                                     R y[V];
                                     load_row<V>(rg + (B - 1 - b + g) * P + jb * V, y);
 #pragma unroll
@@ -924,7 +998,7 @@ __global__ void __launch_bounds__(32 * kNearWarps, B == 1 ? 6 : sizeof(H) == 8 ?
                 for (int b = 0; b < B; ++b) tot[b] = wide(acc[b] * ks) + (iters > 4 ? mid[b * 32 + lane] : 0.0);
             }
         }
-    } else if constexpr (sizeof(H) != 2) {   // (those of FP16 plans go to the FP32 instance)
+    } else if constexpr (sizeof(H) != 2 || B == 1) {   // (those of a block of FP16 plans go to the FP32 instance)
         // aux slices: slice 0 the static tile (times C_j(n - W), it carries dt), slice 1 + q the tail
         // coefficients of term q (times the tail state V_qj(n) = rho_q V_qj(n - 1) + D_{j, n-W}, updated
         // here by its only reader).  Lane j of a lane group forms its slice's rows of the B steps.

@@ -47,8 +47,8 @@ __device__ __forceinline__ void mma_16816_first(float (&c)[4], unsigned a0, unsi
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
-// NR right-hand sides, B steps of a launch (1 or 16).  Rows in shared memory: row q of the item holds the slip
-// rates of step n + S - 1 - k0 - q, S the steps rounded up to whole tiles, [q][part][right-hand side][32 sources] with
+// NR right-hand sides, a block of steps.  Rows in shared memory: row q of the item holds the slip
+// rates of step n + S - 1 - k0 - q, S = kBlk, [q][part][right-hand side][32 sources] with
 // the parts hi, lo; 8 consecutive rows are the columns of one MMA tile, so window slice k takes the tiles from
 // row k - k0 on (tile = one step of 8 right-hand sides' hi or lo, of 4 with both, 2 steps of 2).
 //
@@ -65,24 +65,23 @@ __device__ __forceinline__ void mma_16816_first(float (&c)[4], unsigned a0, unsi
 // sides of N = 2500 from 1.36 to 1.53 ms.)
 static const int kSum = 8;
 
-template <int NR, int B>
+template <int NR>
 struct TcCfg {
     static constexpr int C = 2 * NR;                          // columns of one row q
     static constexpr int per = NR == 2 ? 2 : 1;               // steps of one tile
-    static constexpr int S = B < per ? per : B;
-    static constexpr int tiles = S / per;                     // accumulator tiles (hi and lo of 8 share one)
-    static constexpr int warps = B == 1 ? 2 : 4;
-    static constexpr int share = B == 1 ? 1 : tiles / 2;      // tiles of a warp at most
-    static constexpr int rows(int chunk) { return chunk + S - 1; }
+    static constexpr int tiles = kBlk / per;                  // accumulator tiles (hi and lo of 8 share one)
+    static constexpr int warps = 4;
+    static constexpr int share = tiles / 2;                   // tiles of a warp at most
+    static constexpr int rows(int chunk) { return chunk + kBlk - 1; }
     static constexpr size_t row_bytes(int chunk) { return (size_t)rows(chunk) * C * 64; }
     // rows and their scales
     static constexpr size_t smem(int chunk) { return row_bytes(chunk) + (size_t)rows(chunk) * C * 4; }
 };
 
-template <int NR, int B>
-__global__ void __launch_bounds__(32 * TcCfg<NR, B>::warps, B == 1 ? 8 : 4) tc_block_kernel(StepArgs<float> a, int chunk) {
-    using Cf = TcCfg<NR, B>;
-    constexpr int C = Cf::C, S = Cf::S, NW = Cf::warps, T = Cf::share;
+template <int NR>
+__global__ void __launch_bounds__(32 * TcCfg<NR>::warps, 4) tc_block_kernel(StepArgs<float> a, int chunk) {
+    using Cf = TcCfg<NR>;
+    constexpr int C = Cf::C, S = kBlk, NW = Cf::warps, T = Cf::share;
     extern __shared__ __align__(16) unsigned char tc_smem[];
     const NearTask tk = a.tasks[blockIdx.x];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -127,12 +126,11 @@ __global__ void __launch_bounds__(32 * TcCfg<NR, B>::warps, B == 1 ? 8 : 4) tc_b
     }
     __syncthreads();
     // this warp's receivers 16 mt ... 16 mt + 15 and tiles i0 ... i0 + nt - 1 (leaves of at most 16 receivers
-    // have one set of receivers: a quarter of the tiles per warp; one step: the second warp has nothing to do)
+    // have one set of receivers: a quarter of the tiles per warp)
     const bool two = nr > 16;
     const int mt = two ? warp & 1 : 0;
-    const int nt = B == 1 ? (two || warp == 0 ? 1 : 0) : two ? T : T / 2;
-    const int i0 = B == 1 ? 0 : (two ? warp >> 1 : warp) * nt;
-    if (!nt) return;
+    const int nt = two ? T : T / 2;
+    const int i0 = (two ? warp >> 1 : warp) * nt;
     const int g = lane >> 2, t = lane & 3;
     // the 16-byte vectors (sources 8 t ... 8 t + 7) of receivers g and g + 8 of the set
     const __half* base = (const __half*)a.tensor + tk.off + ((size_t)t * nr + 16 * mt + g) * 8;
@@ -213,4 +211,123 @@ __global__ void __launch_bounds__(32 * TcCfg<NR, B>::warps, B == 1 ? 8 : 4) tc_b
             if (mine && fits && b < nb && 16 * mt + row < nr) out[r * a.rs_partial + b * a.cap_partial + row] = wide(v * ks);
         }
     }
+}
+
+// One step of NR right-hand sides: a slip-rate row meets one slice only, so the lanes split it in registers, each the
+// eight sources 8 t ... 8 t + 7 of its column g that are its B fragment.  One warp per item, both sets of receivers;
+// the sums of the block kernel, bit for bit.  (The block kernel's way, through shared memory, took 40 instructions a row
+// and right-hand side where this takes 10: eight right-hand sides, N = 6000, 642 us against 272 a step; 490 us with the
+// rows split once for all leaves that share them, which loses digits where a leaf is quiet.)
+static const int kTcStepWarps = 4;
+
+template <int NR>
+__global__ void __launch_bounds__(32 * kTcStepWarps, 4) tc_step_kernel(StepArgs<float> a, int n_win) {
+    const int it = blockIdx.x * kTcStepWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (it >= n_win) return;   // warp-uniform
+    const NearTask tk = a.tasks[it];
+    const int n = step_index(a), nr = tk.nr, ns = tk.ns;
+    const int nk = tk.k0 <= n ? tk.k1 - tk.k0 : 0;   // (0: the item's window lies before the march)
+    const int g = lane >> 2, t = lane & 3;
+    const int r = g % NR;                            // column g: right-hand side r,
+    const bool low = NR < 8 && g / NR % 2;           // hi or lo (8 right-hand sides: both, one MMA after the other)
+    const __half* base = (const __half*)a.tensor + tk.off + ((size_t)t * nr + g) * 8;
+    const bool in = FDPH_IDX(tk.off + (long long)nk * tk.sl <= a.len_tensor, a.err) && 8 * t < ns;
+    const int top = n - tk.k0, hend = hist_end(a, n), stop = wrap(top, a.WD);
+    const float* ring = a.Dring32 + r * a.rs_D + tk.s0 + 8 * t;
+    constexpr int D = 2;   // slices in flight
+    uint4 xn[D][4];        // receivers g, g + 8, g + 16, g + 24
+    float yn[D][8];
+    auto load = [&](int k, uint4 (&x)[4], float (&y)[8]) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            x[m] = in && k < nk && g + 8 * m < nr ? __ldcs((const uint4*)(base + (size_t)k * tk.sl + 64 * m)) : make_uint4(0, 0, 0, 0);
+        const int tt = top - k;
+        int slot = stop - k;   // nk <= WD: one wrap at most
+        slot += slot < 0 ? a.WD : 0;
+        const bool ok = k < nk && tt >= 0 && tt < hend;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y[i] = ok && 8 * t + i < ns ? ring[(size_t)slot * a.N + i] : 0.f;
+    };
+#pragma unroll
+    for (int d = 0; d < D; ++d) load(d, xn[d], yn[d]);
+    float acc[2][4], sum[2][4];
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) acc[m][f] = sum[m][f] = 0.f;
+    for (int k = 0; k < nk; ++k) {
+        uint4 x[4];
+        float y[8];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) x[m] = xn[0][m];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y[i] = yn[0][i];
+#pragma unroll
+        for (int d = 0; d + 1 < D; ++d) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) xn[d][m] = xn[d + 1][m];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) yn[d][i] = yn[d + 1][i];
+        }
+        load(k + D, xn[D - 1], yn[D - 1]);
+        unsigned big = 0;   // the largest of the column's 32 slip rates: those of lanes 4 g ... 4 g + 3
+#pragma unroll
+        for (int i = 0; i < 8; ++i) big = max(big, __float_as_uint(fabsf(y[i])));
+        big = max(big, __shfl_xor_sync(0xffffffffu, big, 1));
+        big = max(big, __shfl_xor_sync(0xffffffffu, big, 2));
+        const int sh = row_shift(big);
+        const float up = pow2f(sh), down = pow2f(-sh);
+        unsigned hi[4], lo[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float y0 = y[2 * i] * up, y1 = y[2 * i + 1] * up;
+            const __half2 h = __floats2half2_rn(y0, y1);
+            const float2 hf = __half22float2(h);
+            const float z0 = fabsf(y0) <= 65504.f ? y0 - hf.x : 0.f, z1 = fabsf(y1) <= 65504.f ? y1 - hf.y : 0.f;
+            const __half2 l = __floats2half2_rn(z0, z1);   // (an infinity has no rest)
+            hi[i] = *reinterpret_cast<const unsigned*>(&h);
+            lo[i] = *reinterpret_cast<const unsigned*>(&l);
+        }
+        // the scales of columns 2 t and 2 t + 1 (column c: lanes 4 c ...)
+        const float s0 = __shfl_sync(0xffffffffu, down, 8 * t), s1 = __shfl_sync(0xffffffffu, down, 8 * t + 4);
+        unsigned b[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) b[i] = low ? lo[i] : hi[i];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            if (m && nr <= 16) break;   // (warp-uniform)
+            float c[4];
+            mma_16816_first(c, x[2 * m].x, x[2 * m + 1].x, x[2 * m].y, x[2 * m + 1].y, b[0], b[1]);
+            mma_16816(c, x[2 * m].z, x[2 * m + 1].z, x[2 * m].w, x[2 * m + 1].w, b[2], b[3]);
+            if constexpr (NR == 8) {
+                mma_16816(c, x[2 * m].x, x[2 * m + 1].x, x[2 * m].y, x[2 * m + 1].y, lo[0], lo[1]);
+                mma_16816(c, x[2 * m].z, x[2 * m + 1].z, x[2 * m].w, x[2 * m + 1].w, lo[2], lo[3]);
+            }
+            acc[m][0] = fmaf(c[0], s0, acc[m][0]);
+            acc[m][1] = fmaf(c[1], s1, acc[m][1]);
+            acc[m][2] = fmaf(c[2], s0, acc[m][2]);
+            acc[m][3] = fmaf(c[3], s1, acc[m][3]);
+        }
+        if (k % kSum == kSum - 1 || k + 1 == nk) {
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int f = 0; f < 4; ++f) {
+                    sum[m][f] += acc[m][f];
+                    acc[m][f] = 0.f;
+                }
+        }
+    }
+    const bool fits = FDPH_IDX((long long)tk.item * 32 + 32 <= a.cap_partial, a.err);
+    const float ks = a.kinv;   // the window's storage scale (a power of two)
+    double* out = a.partial + (size_t)tk.item * 32;
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            float v = sum[m][f];
+            if constexpr (NR < 8) v += __shfl_xor_sync(0xffffffffu, v, NR / 2);   // hi + lo
+            const int col = 2 * t + (f & 1), row = 16 * m + g + 8 * (f >> 1);
+            if (col < NR && fits && row < nr) out[col * a.rs_partial + row] = wide(v * ks);
+        }
 }
