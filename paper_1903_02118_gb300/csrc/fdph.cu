@@ -611,14 +611,15 @@ static void launch_near(fdph_plan_t P, const StepArgs<T>& a, cudaStream_t s) {
         if (a.nb == 1) launch_near_items<T, double, 1>(a, P->chunk, s);
         else launch_near_items<T, double, kBlk>(a, P->chunk, s);
     } else if (P->precision == FDPH_FP16) {
-        if (!P->n_win) return;
+        const bool all = a.nb == 1 && P->nrhs == 1;   // (see launch_near_aux)
+        if (!P->n_win && !all) return;
         StepArgs<T> w = a;   // (a block of one right-hand side)
         w.n_items = P->n_win;
         switch (P->nrhs) {
             case 2: launch_tc<2>(a, P->n_win, P->chunk, s); break;
             case 4: launch_tc<4>(a, P->n_win, P->chunk, s); break;
             case 8: launch_tc<8>(a, P->n_win, P->chunk, s); break;
-            default: a.nb == 1 ? launch_near_items<T, __half, 1>(a, P->chunk, s) : launch_near_items<T, __half, kBlk>(w, P->chunk, s);
+            default: all ? launch_near_items<T, __half, 1>(a, P->chunk, s) : launch_near_items<T, __half, kBlk>(w, P->chunk, s);
         }
     } else if (a.nb == 1) {
         launch_near_items<T, float, 1>(a, P->chunk, s);
