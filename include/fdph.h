@@ -176,8 +176,8 @@ typedef struct fdph_stats {
     double mean_rank;
     int64_t near_entries;      /* stored kernel coefficients of the inadmissible leaves */
     int64_t far_entries;       /* stored factor / waveform coefficients */
-    int64_t arena_bytes;       /* device bytes of the plan (operator data) */
-    int64_t state_bytes;       /* device bytes of the time-stepping state (rings, accumulators) */
+    int64_t arena_bytes;       /* device bytes of the plan beside state_bytes (operator data, work lists) */
+    int64_t state_bytes;       /* device bytes of the time-stepping state (rings, accumulators) and of a block's scratch */
     double bytes_per_step;     /* algorithmic HBM bytes of one full step at steady state */
     double near_bytes_per_step;/* of which the near-field kernel: coefficients, slip-rate window rows, tail states */
     double flops_per_step;     /* multiply-adds x 2 of one full step */

@@ -325,6 +325,7 @@ struct fdph_plan_s {
     double *ring = nullptr, *zring = nullptr, *partial = nullptr;
     void* dhat = nullptr;
     size_t state_bytes = 0;
+    size_t device_bytes = 0;  // of all allocations
     // host staging for fdph_step_host
     double *dD = nullptr, *dT = nullptr;
     // per-kernel event timing
@@ -389,6 +390,7 @@ static int dalloc(fdph_plan_t P, T** out, size_t count) {
         return FDPH_E_OOM;
     }
     P->allocs.push_back(p);
+    P->device_bytes += bytes + extra;
 #ifdef FDPH_CHECK
     P->canaries.push_back({(unsigned char*)p + bytes, extra});
     if (cudaMemsetAsync((unsigned char*)p + bytes, kCanary, extra, P->stream) != cudaSuccess) return FDPH_E_CUDA;
@@ -1419,10 +1421,7 @@ static void fill_stats(fdph_plan_t P) {
     s.near_bytes_per_step = near_b;
     s.flops_per_step = flops;
     s.state_bytes = (long long)P->state_bytes;
-    long long arena = 0;
-    arena += (long long)(hp.fac.size() * ps) + hp.ints.size() * 4 + hp.sbs.size() * sizeof(SbDev);
-    arena += (long long)(hp.near_tensor_len * pw + hp.near_aux_len * ps);
-    s.arena_bytes = arena;
+    s.arena_bytes = (long long)(P->device_bytes - P->state_bytes);
 }
 
 // Near-field work items of `chunk` kernel steps (1..kChunk): new items, partial slots and
@@ -1813,13 +1812,36 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
     stamp("host plan (admissible blocks)");
     if (rc == -3) return fail(FDPH_E_CAUSALITY);
     if (rc) return fail(FDPH_E_ARG);
+    // the factors on the device leave out the Domain-F waveforms, which the FIR keeps in its own order:
+    // ranges [first, first + length) of hp.fac, and what lies before each
+    std::vector<std::pair<long long, long long>> cut;
+    for (const SubBlock& b : hp.sbs)
+        if (b.kind == SB_F) cut.push_back({(long long)b.h, (long long)b.taps * b.ns});
+    std::sort(cut.begin(), cut.end());
+    cut.erase(std::unique(cut.begin(), cut.end()), cut.end());
+    std::vector<long long> cut_before(1, 0);
+    for (const auto& c : cut) cut_before.push_back(cut_before.back() + c.second);
+    auto place = [&](long long x) {   // of an offset in hp.fac
+        const size_t k = std::upper_bound(cut.begin(), cut.end(), std::make_pair(x, LLONG_MAX)) - cut.begin();
+        return x - cut_before[k] + (k && x < cut[k - 1].first + cut[k - 1].second ? cut[k - 1].second - (x - cut[k - 1].first) : 0);
+    };
+    std::vector<double> fac;
+    fac.reserve(hp.fac.size() - (size_t)cut_before.back());
+    {
+        size_t at = 0;
+        for (const auto& c : cut) {
+            fac.insert(fac.end(), hp.fac.begin() + at, hp.fac.begin() + c.first);
+            at = (size_t)(c.first + c.second);
+        }
+        fac.insert(fac.end(), hp.fac.begin() + at, hp.fac.end());
+    }
     // ---- upload the far-field operator
     std::vector<SbDev> sd(hp.sbs.size());
     for (size_t q = 0; q < sd.size(); ++q) {
         const SubBlock& b = hp.sbs[q];
         const int LH = b.maxdelay - b.mindelay + 1;
         sd[q] = {b.kind, b.rank, b.r0, b.nr, b.s0, b.ns, b.L, b.LZ, b.taps, b.maxdelay, b.mindm, b.run0,
-                 b.soe, b.ident, LH, (long long)b.f, (long long)b.g, (long long)b.h, (long long)b.ring, (long long)b.zring,
+                 b.soe, b.ident, LH, place(b.f), place(b.g), b.kind == SB_F ? 0 : place(b.h), (long long)b.ring, (long long)b.zring,
                  (long long)b.dhat, (long long)b.delay, (long long)b.dm, (long long)b.ustate, (long long)b.trc,
                  (long long)b.phi, 0, b.mindelay, b.qn, (long long)b.qb};
     }
@@ -1866,7 +1888,7 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
         const SubBlock& b = hp.sbs[hp.g_sb[e]];
         const int il = hp.g_il[e];
         const bool tr = b.kind == SB_TR;
-        ents[e] = {tr ? (long long)b.zring : (long long)b.ring, b.ident == 1 ? il : (long long)b.f + (long long)il * b.rank,
+        ents[e] = {tr ? (long long)b.zring : (long long)b.ring, b.ident == 1 ? il : place(b.f) + (long long)il * b.rank,
                    tr ? b.LZ : b.L, hp.ints[b.dm + il], b.rank, (tr ? 1 : 0) | (b.ident == 1 ? 2 : 0)};
         if (hp.interp) ephi[e] = hp.phis[b.phi + il];
     }
@@ -1928,7 +1950,7 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
         (rc = upload(P, &P->tr_l, hp.tr_l)) || (rc = upload(P, &P->g_ptr, hp.g_ptr)))
         return fail(rc);
     if (P->precision != FDPH_FP64) {
-        std::vector<float> f(hp.fac.begin(), hp.fac.end());
+        std::vector<float> f(fac.begin(), fac.end());
         float* d = nullptr;
         if ((rc = upload(P, &d, f))) return fail(rc);
         P->fac = d;
@@ -1938,7 +1960,7 @@ int fdph_plan(const fdph_geometry* geometry, const fdph_material* material, doub
         P->fir_h = dh;
     } else {
         double* d = nullptr;
-        if ((rc = upload(P, &d, hp.fac))) return fail(rc);
+        if ((rc = upload(P, &d, fac))) return fail(rc);
         P->fac = d;
         double* dh = nullptr;
         if ((rc = upload(P, &dh, fh))) return fail(rc);

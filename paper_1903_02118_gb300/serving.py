@@ -5,13 +5,12 @@ admitted as soon as its device footprint (plan operator + time-stepping state + 
 the HBM budget and a slot is free; admitted scenarios stay resident and all of them advance
 together, each iteration moving every live scenario forward by `chunk` time steps: the
 scenarios with a full chunk ahead as one batch (fdph_batch_rupture_run: every plan's blocks of
-steps on the plan's own stream), the others (a last, shorter chunk) with their own step graphs
-on their own CUDA streams.  A finished scenario releases its memory at once and the next
+steps on the plan's own stream), the others (a last, shorter chunk) each on its own CUDA stream.  A finished scenario releases its memory at once and the next
 waiting request takes its place.  Per request the loop records queueing, plan and run times and
 the time to solution (arrival to last step on the device).
 
 All arithmetic runs in libfdph (fdph_plan, fdph_rupture_init, fdph_batch_rupture_run,
-fdph_rupture_run: captured step graphs replayed per chunk); this module only schedules, and
+fdph_rupture_run: captured blocks of steps replayed per chunk); this module only schedules, and
 builds plans on background threads so that planning overlaps the stepping of the live
 scenarios.  Plans are independent, so a scenario's result is bit-identical alone and in the mix
 (tests/test_gpu_serving.py).
@@ -88,8 +87,8 @@ class Server:
         self.time_scale = time_scale
         self.planners = planners
         self.precision = precision
-        # batch=True: live scenarios with a full chunk ahead step together, one near-field launch
-        # per step for all of them (fdph_batch_rupture_run); otherwise each on its own stream
+        # batch=True: live scenarios with a full chunk ahead step together (fdph_batch_rupture_run, which
+        # orders the plans' streams around the call); otherwise each on its own stream
         self.batch = batch
         self._batch, self._batch_key = None, None
         # each planner builds with its share of the host cores (the builds run at the same time)
@@ -246,9 +245,10 @@ def footprint_model(xy, dt, M, eta=0.5, leaf=32, precision=fdph.FP32, soe_terms=
     coefficients (v = 16 bytes / element), W = the leaf's longest wave passage (farthest end point
     over c dt) + n_c with exponential tails (the whole march M when too little is left to fit a
     tail), or + the steps the remainder takes to decay to eps_st without them (the paper's cut),
-    + the static and tail slices; the admissible blocks add their factors and rings
-    (5 low-rank operators per leaf at `rank`, ring slots up to the largest delay); the state adds the
-    slip-rate rings, and the serving loop its chunk buffers."""
+    + the static and tail slices, the tails' FP64 projections and the partial sums of a block's 16 steps (4 KB per
+    work item of about 16 slices); the admissible blocks add their factors and rings (5 low-rank operators per
+    leaf at `rank`, ring slots up to the largest delay); the state adds the slip-rate rings with their room
+    for a block and a block's rows, and the serving loop its chunk buffers."""
     tx = fdph.tree_export(xy, dt, eta=eta, leaf_size=leaf, extra_steps=-1)
     perm = tx["perm"]
     N = xy.shape[0]
@@ -276,10 +276,11 @@ def footprint_model(xy, dt, M, eta=0.5, leaf=32, precision=fdph.FP32, soe_terms=
             wmax = max(wmax, W)
             v = 16 // sw
             near += W * (-(-lf["ns"] // v) * v) * lf["nr"] * sw + (1 + soe_terms) * (-(-lf["ns"] // 4) * 4) * lf["nr"] * sa
+            near += 8 * soe_terms * lf["nr"] * lf["ns"] + 4096 * (-(-W // 16) + 2)
         else:
             L = int(np.max(lf["mbar"]) + np.max(lf["Dm"]) + np.max(lf["dm"]) - np.min(lf["dm"])) + 2
             far += 5 * rank * ((lf["nr"] + lf["ns"]) * sa + 8 * L) + 4 * (lf["nr"] + 2 * lf["ns"])
-    state = (wmax + 1) * N * (8 + 4) + 2 * (wmax + 1) * N * 8 + 16 * N * 8
+    state = (wmax + 16) * N * (8 + 4) + 2 * (wmax + 16) * N * 8 + 16 * N * 8 * 4
     return int(near + far + state + 3 * N * 8 * (chunk + 2))
 
 
