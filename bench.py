@@ -436,8 +436,9 @@ def near_roofline(plan, st, Dd, Td, n_from, K, hbm_peak):
     plan.set_profiling(False)
     near_ms = kt["near"][0] / max(kt["near"][1], 1)
     achieved = st["near_bytes_per_step"] * -(-K // 16) / K / (near_ms * 1e-3) / 1e9
+    tc = plan.precision == 2 and plan.nrhs > 1   # (FP16 windows of several right-hand sides)
     return kt, {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
-                "kernel": "near_block_kernel", "kernel_ms": {k: v[0] / max(v[1], 1) for k, v in kt.items()}}
+                "kernel": "tc_block_kernel" if tc else "near_block_kernel", "kernel_ms": {k: v[0] / max(v[1], 1) for k, v in kt.items()}}
 
 
 def rel_err(T, T_or, rows):

@@ -1,14 +1,15 @@
 // fdph.cu -- device side of the FDP=H time step and the C ABI (include/fdph.h).
 //
-// Steps run in blocks of up to 16 (step.cuh); the kernels of a block are captured as one CUDA graph: FIR +
-// scatter and transient + Eq. 39 on two side streams, beside the near field, all joined before the gather.
-// Causality (min(dm + delay) >= 1, checked at plan time) guarantees that the ring slots read at step n were
-// completed by steps < n and that the slots written at step n are not read; where min(dm + delay) is less
-// than the block's length, Eq. 39 follows the scatter.  The near field runs on the CUDA cores (FP64, FP32, and
-// FP16 windows of one right-hand side, step.cuh) or on the tensor cores (FP16 windows of several, tensor.cuh).  Several right-hand
-// sides go through one launch.  A rupture block (Sec. 6.2) takes what the slip rates before the block do to
-// all its steps at once, then step by step its own part, the friction law and the push, then commits the
-// block.  A batch runs its plans on their own streams.
+// Steps run in blocks of up to 16 (step.cuh), a launch per kernel and block: FIR + scatter and transient + Eq. 39
+// on two side streams, beside the near field, all joined before the gather.  (Whole rupture blocks, and the
+// steps of the delayed-history form, replay a captured graph.)  Causality (min(dm + delay) >= 1, checked at plan
+// time) guarantees that the ring slots read at step n were completed by steps < n and that the slots written
+// at step n are not read; where min(dm + delay) is less than the block's length, Eq. 39 follows the scatter.
+// The near field runs on the CUDA cores (FP64, FP32, and FP16 windows of one right-hand side, step.cuh) or on the
+// tensor cores (FP16 windows of several, tensor.cuh).  Several right-hand sides go through one launch.  A rupture
+// block (Sec. 6.2) takes what the slip rates before the block do to all its steps at once, then step by step its
+// own part, the friction law and the push, then commits the block.  A batch runs its plans on their own
+// streams, ordered with one another around each call.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -560,11 +561,12 @@ static void launch_eq42(const StepArgs<T>& a, cudaStream_t s) {
         if (a.n_gat) hgather_kernel<T><<<dim3(blocks((long long)a.n_gat * 32, 128), a.nrhs), 128, 0, s>>>(a);
     } else if (a.n_sct) {
         const int g = blocks((long long)a.n_sct * 32, 128);
-        switch (a.nb == 1 ? a.nrhs : 1) {
-            case 2: scatter_kernel<T, 2><<<g, 128, 0, s>>>(a); break;
-            case 4: scatter_kernel<T, 4><<<g, 128, 0, s>>>(a); break;
-            case 8: scatter_kernel<T, 8><<<g, 128, 0, s>>>(a); break;
-            default: scatter_kernel<T, 1><<<dim3(g, a.nrhs), 128, 0, s>>>(a);
+        switch (a.nb == 1 ? a.nrhs : 0) {
+            case 1: scatter_kernel<T, 1, true><<<g, 128, 0, s>>>(a); break;
+            case 2: scatter_kernel<T, 2, true><<<g, 128, 0, s>>>(a); break;
+            case 4: scatter_kernel<T, 4, true><<<g, 128, 0, s>>>(a); break;
+            case 8: scatter_kernel<T, 8, true><<<g, 128, 0, s>>>(a); break;
+            default: scatter_kernel<T, 1, false><<<dim3(g, a.nrhs), 128, 0, s>>>(a);
         }
     }
 }

@@ -140,7 +140,7 @@ extern "C" int fdph_plain_step_noalloc(const double* K, int32_t n, int32_t W, co
     nsplit = std::max(1LL, std::min(nsplit, FDPH_NOALLOC_MAX_PARTIALS / (tiles * kTile)));
     noalloc_partial_kernel<<<(unsigned)(tiles * nsplit), kThreads, 0, s>>>(K, n, rows, D_hist, hist_len, step, (int)nsplit,
                                                                            partial);
-    // the reduction is launched while the sums are under way (it waits for them on the device)
+    // the reduction's launch does not wait for the sums to end: its CTAs start as theirs exit, and wait on the device
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(((long long)n * 32 + kThreads - 1) / kThreads));
     cfg.blockDim = dim3(kThreads);

@@ -472,10 +472,10 @@ __global__ void __launch_bounds__(32 * kFirWarps) fir_step_kernel(StepArgs<T> a,
 // ---- Eq. 42
 
 // source quantity u_j of Eq. 42 of the block's b-th step: Dhat (Domain F), dt * cumulative slip
-// (Domain S, App. B.1), slip rate (transient); of a single step, of right-hand side r past the arguments' own
+// (Domain S, App. B.1), slip rate (transient); of a single step, of right-hand side r past the arguments' own.
+// pitch: blk_pitch(a), where it is not known when the kernel is compiled
 template <class T>
-__device__ __forceinline__ double source_value(const StepArgs<T>& a, const SbDev& sb, int jl, int b, int r = 0) {
-    const int pitch = blk_pitch(a);
+__device__ __forceinline__ double source_value(const StepArgs<T>& a, const SbDev& sb, int jl, int pitch, int b, int r = 0) {
     if (sb.kind == 0) return wide(a.dhat[(sb.dhat + jl) * pitch + b + r]);
     return (sb.kind == 1 ? a.blkC : a.blkD)[(size_t)(sb.s0 + jl) * pitch + b + r];
 }
@@ -485,9 +485,10 @@ __device__ __forceinline__ double source_value(const StepArgs<T>& a, const SbDev
 // brings one of the block's steps there, oldest step first.  2^lg lanes per slot cover the rank
 // index, so the slots of a warp are one contiguous piece of the ring, read and written once per
 // block (a step-by-step scatter updates a slot once for every source).
-// NR right-hand sides in one lane (one step: the factors are read once), or one per grid row (blocks).
-template <class T, int NR>
+// NR right-hand sides in one lane (kOne, one step: the factors are read once), or one per grid row (blocks).
+template <class T, int NR, bool kOne>
 __global__ void scatter_kernel(StepArgs<T> a0) {
+    constexpr int pitch = kOne ? NR : kBlk;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const StepArgs<T> a = rhs_args(a0, blockIdx.y);
     if (w >= a.n_sct) return;
@@ -514,7 +515,7 @@ __global__ void scatter_kernel(StepArgs<T> a0) {
                 const int jl = a.src_order[rn.z + u];
                 if (!FDPH_IDX(jl < rank, a.err)) continue;
 #pragma unroll
-                for (int r = 0; r < NR; ++r) ring[r * a.len_ring + jl] = source_value(a, sb, jl, b, r);
+                for (int r = 0; r < NR; ++r) ring[r * a.len_ring + jl] = source_value(a, sb, jl, pitch, b, r);
             }
         }
         return;
@@ -532,7 +533,7 @@ __global__ void scatter_kernel(StepArgs<T> a0) {
             if (rn.y == 1) {
                 const double gl = wide(g[(long long)rn.w * rank + l]);
 #pragma unroll
-                for (int r = 0; r < NR; ++r) v[r] = fma(gl, source_value(a, sb, rn.w, b, r), v[r]);
+                for (int r = 0; r < NR; ++r) v[r] = fma(gl, source_value(a, sb, rn.w, pitch, b, r), v[r]);
             } else {
                 double s[NR];
 #pragma unroll
@@ -541,7 +542,7 @@ __global__ void scatter_kernel(StepArgs<T> a0) {
                     const int jl = a.src_order[rn.z + u];
                     const double gl = wide(g[(long long)jl * rank + l]);
 #pragma unroll
-                    for (int r = 0; r < NR; ++r) s[r] = fma(gl, source_value(a, sb, jl, b, r), s[r]);
+                    for (int r = 0; r < NR; ++r) s[r] = fma(gl, source_value(a, sb, jl, pitch, b, r), s[r]);
                 }
 #pragma unroll
                 for (int r = 0; r < NR; ++r) v[r] += s[r];
@@ -565,7 +566,7 @@ __global__ void record_kernel(StepArgs<T> a0) {
     if (q >= a.n_rec) return;
     const int2 t = a.rec_tasks[q];
     const SbDev& sb = a.sbs[t.x];
-    a.uhist[sb.uhist + (long long)wrap(step_index(a), sb.LH) * sb.ns + t.y] = source_value(a, sb, t.y, 0);
+    a.uhist[sb.uhist + (long long)wrap(step_index(a), sb.LH) * sb.ns + t.y] = source_value(a, sb, t.y, blk_pitch(a), 0);
 }
 
 // one warp per (block, rank index l), lanes over the sources
