@@ -55,8 +55,8 @@ METRIC_REL_ERR = 1e-4      # the metric's accuracy condition (relative error vs 
 # near-field coefficient: the near bytes scale with the stored coefficients, so a full launch's
 # traffic is this figure times the plan's coefficients.  Reported only while the near-field
 # kernel's source (near_kernel_source_hash) is the one that was captured.
-NEAR_NCU = {"source_sha256": "b8e0626781aed8c333d157ee8d30181af24daae8ddebe2f261d6f2d908deb1aa",
-            "dram_bytes_per_coefficient": 1.453, "precision": 1, "nrhs": 1,
+NEAR_NCU = {"source_sha256": "556658d00d134d04a14f8f8a79317e46093c9e22aec67f3515180582af187e87",
+            "dram_bytes_per_coefficient": 1.456, "precision": 1, "nrhs": 1,
             "capture": "profiles/block_kernels_curved_n2048_m1024.md (curved N = 2048, M = 1024, FP32, "
                        "Q = 16, one launch of 16 steps)"}
 
