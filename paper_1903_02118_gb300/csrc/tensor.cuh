@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(32 * TcCfg<NR>::warps, 4) tc_block_kernel(Step
 // One step of NR right-hand sides: a slip-rate row meets one slice only, so the lanes split it in registers, each the
 // eight sources 8 t ... 8 t + 7 of its column g that are its B fragment.  One warp per item, both sets of receivers;
 // the sums of the block kernel, bit for bit.  (The block kernel's way, through shared memory, took 40 instructions a row
-// and right-hand side where this takes 10: eight right-hand sides, N = 6000, 642 us against 272 a step; 490 us with the
+// and right-hand side where this takes 10: eight right-hand sides, N = 6000, 479 us against 272 a step; 490 us with the
 // rows split once for all leaves that share them, which loses digits where a leaf is quiet.)
 static const int kTcStepWarps = 4;
 
